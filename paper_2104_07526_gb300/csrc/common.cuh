@@ -18,7 +18,7 @@
 // culled slots drop out at the one visibility test.  The compiler can then
 // interleave the divisions of a lane's slots.
 //
-// project_pair computes the same results for two slots at once (see there):
+// project_slots computes the same results for a lane's slots, two at a time:
 // Blackwell's paired float32 instructions (each half rounded on its own, as
 // the scalar instruction rounds it) for the matrix rows and the screen
 // transform, and one reciprocal per slot shared by both screen divisions,
@@ -99,23 +99,30 @@ __device__ __forceinline__ f32x2 f2_fma(f32x2 a, f32x2 b, f32x2 c) {
   return r;
 }
 
-__device__ __forceinline__ float add_rn(float a, float b) {
-  float r;
-  asm("add.rn.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+__device__ __forceinline__ f32x2 f2_add(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
   return r;
 }
 
-// One matrix row for two slots: the three products as paired instructions,
-// the sums as scalar add.rn on the halves.  Paired sums are not used: ptxas
-// fuses a paired product into a following paired add (or into fma with a
-// factor of one) despite the .rn modifier, which would change roundings.
-// A scalar add.rn is never fused.
-__device__ __forceinline__ f32x2 row_dot2(const float r[4], f32x2 x, f32x2 y, f32x2 z) {
-  float a0, b0, a1, b1, a2, b2;
-  f2_unpack(f2_mul(f2_bcast(r[0]), x), a0, b0);
-  f2_unpack(f2_mul(f2_bcast(r[1]), y), a1, b1);
-  f2_unpack(f2_mul(f2_bcast(r[2]), z), a2, b2);
-  return f2_pack(add_rn(add_rn(add_rn(a0, a1), a2), r[3]), add_rn(add_rn(add_rn(b0, b1), b2), r[3]));
+// -0 in both halves, from a value (a viewport size, positive) that the
+// assembler cannot know.
+__device__ __forceinline__ f32x2 f2_opaque_neg_zero(float positive) {
+  return f2_bcast(__uint_as_float((__float_as_uint(positive) & 0x80000000u) ^ 0x80000000u));
+}
+
+// One matrix row for two slots, every product and sum rounded on its own.
+// A product is written as a fused multiply-add of -0, which rounds as the
+// product does (and keeps its sign when it is zero): ptxas fuses a plain
+// paired product into a following paired add despite the .rn modifier, which
+// would change roundings, but it has no operation for the sum of a fused
+// multiply-add and another value.  `nz` must not be a constant it can see.
+// Six instructions a row for two slots; nine with scalar sums.
+__device__ __forceinline__ f32x2 row_dot2(const float r[4], f32x2 x, f32x2 y, f32x2 z, f32x2 nz) {
+  const f32x2 a = f2_fma(f2_bcast(r[0]), x, nz);
+  const f32x2 b = f2_fma(f2_bcast(r[1]), y, nz);
+  const f32x2 c = f2_fma(f2_bcast(r[2]), z, nz);
+  return f2_add(f2_add(f2_add(a, b), c), f2_bcast(r[3]));
 }
 
 // Hardware reciprocal estimate (within 1 ulp of 1/w).
@@ -128,11 +135,10 @@ __device__ __forceinline__ float rcp_estimate(float w) {
 // w for which the reciprocal path below is exact: [2^-40, 2^40).  Every
 // quantity it forms is then a normal number or an exact zero, or the point
 // is culled either way (below).
-constexpr uint32_t kRcpWindowLo = 0x2B800000u;                  // bits of 2^-40
-constexpr uint32_t kRcpWindowSpan = 0x53800000u - kRcpWindowLo;  // up to bits of 2^40
+constexpr float kRcpWindowBottom = 0x1p-40f, kRcpWindowTop = 0x1p40f;
 
 __device__ __forceinline__ bool in_rcp_window(float w) {
-  return __float_as_uint(w) - kRcpWindowLo < kRcpWindowSpan;
+  return w >= kRcpWindowBottom && w < kRcpWindowTop;
 }
 
 // RN(1/w) for both halves: one Newton step with fused operations on the
@@ -156,62 +162,85 @@ __device__ __forceinline__ f32x2 quotient2(f32x2 c, f32x2 nw, f32x2 y) {
   return f2_fma(f2_fma(q0, nw, c), y, q0);
 }
 
-// project() for slots a and b: the same results, bit for bit.  The matrix
-// rows are summed in the same order with the same roundings; the screen
-// transform is the same fused multiply-add and product; each quotient equals
-// the IEEE one (quotient2).  A slot whose w is valid but outside the window
-// takes the IEEE divisions.  pa / pb are meaningful only when va / vb.
-__device__ __forceinline__ void project_pair(const ViewParams& v, const uint4& ra, const uint4& rb, uint32_t& pa,
-                                             uint32_t& pb, float& wa, float& wb, bool& va, bool& vb) {
-  const f32x2 x = f2_pack(__uint_as_float(ra.x), __uint_as_float(rb.x));
-  const f32x2 y = f2_pack(__uint_as_float(ra.y), __uint_as_float(rb.y));
-  const f32x2 z = f2_pack(__uint_as_float(ra.z), __uint_as_float(rb.z));
-  const f32x2 w2 = row_dot2(v.r3, x, y, z);
-  const f32x2 cx = row_dot2(v.r0, x, y, z);
-  const f32x2 cy = row_dot2(v.r1, x, y, z);
-  f2_unpack(w2, wa, wb);
-  const f32x2 nw = f2_mul(w2, f2_bcast(-1.0f));
-  const f32x2 rw = reciprocal2(nw, wa, wb);
-  float sxa, sxb, sya, syb;
-  f2_unpack(f2_mul(f2_fma(quotient2(cx, nw, rw), f2_bcast(0.5f), f2_bcast(0.5f)), f2_bcast(v.fw)), sxa, sxb);
-  f2_unpack(f2_mul(f2_fma(quotient2(cy, nw, rw), f2_bcast(0.5f), f2_bcast(0.5f)), f2_bcast(v.fh)), sya, syb);
-  const bool oka = __float_as_uint(wa) - 1u < 0x7F7FFFFFu;
-  const bool okb = __float_as_uint(wb) - 1u < 0x7F7FFFFFu;
-  const bool slowa = oka && !in_rcp_window(wa);
-  const bool slowb = okb && !in_rcp_window(wb);
-  if (slowa || slowb) {
-    float cxa, cxb, cya, cyb;
-    f2_unpack(cx, cxa, cxb);
-    f2_unpack(cy, cya, cyb);
-    if (slowa) {
-      sxa = to_screen(cxa, wa, v.fw);
-      sya = to_screen(cya, wa, v.fh);
-    }
-    if (slowb) {
-      sxb = to_screen(cxb, wb, v.fw);
-      syb = to_screen(cyb, wb, v.fh);
-    }
-  }
-  const uint32_t bw = __float_as_uint(v.fw), bh = __float_as_uint(v.fh);
-  va = oka && __float_as_uint(sxa) < bw && __float_as_uint(sya) < bh;
-  vb = okb && __float_as_uint(sxb) < bw && __float_as_uint(syb) < bh;
-  pa = __float2uint_rd(sxa) + __float2uint_rd(sya) * v.width;
-  pb = __float2uint_rd(sxb) + __float2uint_rd(syb) * v.width;
+// A positive w outside the window, zero or infinity among two slots.  Where
+// this is false, w is valid exactly when it is positive: a NaN gives false
+// here and is culled by that test.
+__device__ __forceinline__ bool leaves_window(float most, float least_magnitude) {
+  return most >= kRcpWindowTop || least_magnitude < kRcpWindowBottom;
 }
 
-// Every slot of a chunk: pairs, then a last single slot when U is odd.
-// pix[u] is meaningful only when vis[u].
-template <int U>
+// Screen coordinates of two slots from their clip coordinates and w, with the
+// one reciprocal each.
+__device__ __forceinline__ void screen_pair(const ViewParams& v, f32x2 cx, f32x2 cy, const float (&w)[2],
+                                            float (&sx)[2], float (&sy)[2]) {
+  const f32x2 nw = f2_mul(f2_pack(w[0], w[1]), f2_bcast(-1.0f));
+  const f32x2 rw = reciprocal2(nw, w[0], w[1]);
+  const f32x2 half = f2_bcast(0.5f);
+  f2_unpack(f2_mul(f2_fma(quotient2(cx, nw, rw), half, half), f2_bcast(v.fw)), sx[0], sx[1]);
+  f2_unpack(f2_mul(f2_fma(quotient2(cy, nw, rw), half, half), f2_bcast(v.fh)), sy[0], sy[1]);
+}
+
+// project() for U slots (even U): the same results, bit for bit.  The matrix
+// rows are summed in the same order with the same roundings; the screen
+// transform is the same fused multiply-add and product; each quotient equals
+// the IEEE one (quotient2).  A slot whose w leaves the window takes the IEEE
+// divisions, with its pair, or with ONE_TEST (which forms every w first) with
+// all slots of the lane.  ONE_TEST saves instructions where the records die
+// with the projection: the 800M-point key frame takes 1.852 ms with it and
+// 1.869 without, HQS1R (whose records' colours live on) 0.615 and 0.593 ms at
+// 100M points, the 8 x 8 batch 21.98 and 21.70 ms.  (With scalar sums and a
+// test per slot they took 1.888, 0.609 and 22.21 ms.)  pix[u] is meaningful
+// only when vis[u].
+template <int U, bool ONE_TEST = false>
 __device__ __forceinline__ void project_slots(const ViewParams& v, const uint4 (&r)[U], uint32_t (&pix)[U],
                                               float (&w)[U], bool (&vis)[U]) {
+  static_assert(U % 2 == 0, "slots project in pairs");
+  const f32x2 nz = f2_opaque_neg_zero(v.fw);
+  const uint32_t bw = __float_as_uint(v.fw), bh = __float_as_uint(v.fh);
+  auto x = [&](int u) { return f2_pack(__uint_as_float(r[u].x), __uint_as_float(r[u + 1].x)); };
+  auto y = [&](int u) { return f2_pack(__uint_as_float(r[u].y), __uint_as_float(r[u + 1].y)); };
+  auto z = [&](int u) { return f2_pack(__uint_as_float(r[u].z), __uint_as_float(r[u + 1].z)); };
+  if constexpr (ONE_TEST) {
+    float most = 0.0f, least = kRcpWindowTop;
 #pragma unroll
-  for (int u = 0; u + 1 < U; u += 2)
-    project_pair(v, r[u], r[u + 1], pix[u], pix[u + 1], w[u], w[u + 1], vis[u], vis[u + 1]);
-  if constexpr (U % 2 == 1) {
-    pix[U - 1] = 0;
-    w[U - 1] = 0.0f;
-    vis[U - 1] = project(v, __uint_as_float(r[U - 1].x), __uint_as_float(r[U - 1].y), __uint_as_float(r[U - 1].z),
-                         pix[U - 1], w[U - 1]);
+    for (int u = 0; u < U; u += 2) {
+      f2_unpack(row_dot2(v.r3, x(u), y(u), z(u), nz), w[u], w[u + 1]);
+      most = fmaxf(fmaxf(most, w[u]), w[u + 1]);
+      least = fminf(fminf(least, fabsf(w[u])), fabsf(w[u + 1]));
+    }
+    if (__builtin_expect(leaves_window(most, least), 0)) {
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        pix[u] = 0;
+        vis[u] = project(v, __uint_as_float(r[u].x), __uint_as_float(r[u].y), __uint_as_float(r[u].z), pix[u], w[u]);
+      }
+      return;
+    }
+  }
+#pragma unroll
+  for (int u = 0; u < U; u += 2) {
+    if constexpr (!ONE_TEST) f2_unpack(row_dot2(v.r3, x(u), y(u), z(u), nz), w[u], w[u + 1]);
+    const f32x2 cx = row_dot2(v.r0, x(u), y(u), z(u), nz);
+    const f32x2 cy = row_dot2(v.r1, x(u), y(u), z(u), nz);
+    float sx[2], sy[2];
+    screen_pair(v, cx, cy, {w[u], w[u + 1]}, sx, sy);
+    if constexpr (!ONE_TEST) {
+      if (__builtin_expect(leaves_window(fmaxf(w[u], w[u + 1]), fminf(fabsf(w[u]), fabsf(w[u + 1]))), 0)) {
+        float ex[2], ey[2];
+        f2_unpack(cx, ex[0], ex[1]);
+        f2_unpack(cy, ey[0], ey[1]);
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+          sx[k] = w[u + k] < __uint_as_float(kInfBits) ? to_screen(ex[k], w[u + k], v.fw) : -1.0f;  // infinity: culled
+          sy[k] = to_screen(ey[k], w[u + k], v.fh);
+        }
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      vis[u + k] = w[u + k] > 0.0f && __float_as_uint(sx[k]) < bw && __float_as_uint(sy[k]) < bh;
+      pix[u + k] = __float2uint_rd(sx[k]) + __float2uint_rd(sy[k]) * v.width;
+    }
   }
 }
 

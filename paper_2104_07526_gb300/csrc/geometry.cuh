@@ -125,10 +125,6 @@ __device__ __forceinline__ bool slot_in_range(uint32_t base, int u, uint32_t n, 
   }
 }
 
-__device__ __forceinline__ bool project_record(const ViewParams& v, const uint4& r, uint32_t& pix, float& w) {
-  return project(v, __uint_as_float(r.x), __uint_as_float(r.y), __uint_as_float(r.z), pix, w);
-}
-
 // ---------------------------------------------------------------------------
 // Sec. 3.1-3.4: basic key render
 // ---------------------------------------------------------------------------

@@ -93,7 +93,7 @@ __global__ void __launch_bounds__(kThreads, kRenderMinBlocks) k_render_basic(con
     uint32_t pix[U];
     float w[U];
     bool vis[U];
-    project_slots<U>(v, r, pix, w, vis);
+    project_slots<U, true>(v, r, pix, w, vis);
 #pragma unroll
     for (int u = 0; u < U; ++u) vis[u] = vis[u] && slot_in_range<U, L>(base, u, n, full);
     debug_check_pixels<U>(v, pix, vis);

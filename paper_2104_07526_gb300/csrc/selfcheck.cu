@@ -1,5 +1,5 @@
 // Device-side check of the screen division the projection uses
-// (common.cuh: reciprocal2, quotient2, project_pair) against the device's own
+// (common.cuh: reciprocal2, quotient2, project_slots) against the device's own
 // IEEE operations.  A diagnostic behind pcr_check_division: nothing on the
 // render path calls it.
 //

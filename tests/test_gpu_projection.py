@@ -83,3 +83,39 @@ def test_check_rejects_bad_arguments(ctx):
         pcr.pcr_check_division(ctx, ONE, 1, c_first=ONE, c_count=4, c_step=0)
     with pytest.raises(pcr.PcrError):
         pcr.pcr_check_division(ctx, ONE, 1, size=0.0)
+
+
+SPECIAL_W = np.array([2.0**-41, np.nextafter(np.float32(2.0**-40), np.float32(0)), 2.0**-40, 2.0**40,
+                      np.nextafter(np.float32(2.0**40), np.float32(0)), 2.0**41, 1e-42, 0.0, -0.0, -(2.0**-41),
+                      -1.0, -(2.0**41), np.inf, -np.inf, np.nan, 3.4e38], dtype=np.float32)
+
+
+@pytest.mark.parametrize("n", (1, 2, 31, 33, 127, 128, 129, 4099))
+@pytest.mark.parametrize("share", (0.02, 0.5, 1.0))
+def test_slots_that_leave_the_window_beside_slots_inside(ctx, oracle, n, share):
+    """w is the z coordinate: a share of the points have a w outside the
+    reciprocal window, zero, infinite or NaN, so lanes mix both kinds.  Key
+    frames test the window once per lane, the depth and colour passes once
+    per pair of slots."""
+    from gpu_helpers import Renderer
+    rng = np.random.default_rng(n)
+    z = rng.uniform(0.5, 4.0, n).astype(np.float32)
+    z = np.where(rng.random(n) < share, rng.choice(SPECIAL_W, n), z).astype(np.float32)
+    scale = np.where(np.isfinite(z), np.clip(z, -1e37, 1e37), 1.0)
+    xy = (rng.uniform(-1.2, 1.2, (n, 2)) * scale[:, None]).astype(np.float32)
+    cloud = np.empty((n, 4), dtype=np.int32)
+    cloud[:, :2], cloud[:, 2], cloud[:, 3] = xy.view(np.int32), z.view(np.int32), rng.integers(0, 1 << 31, n)
+    m = np.eye(4, dtype=np.float32)
+    m[3] = (0, 0, 1, 0)
+    W, H = 37, 23
+    r = Renderer()
+    r.upload(cloud)
+    r.view(m, W, H)
+    expect = oracle.render_basic(cloud, m, W, H)
+    for v in pcr.EXACT_VARIANTS:
+        assert np.array_equal(r.render_basic(v), expect), v
+    hq = oracle.render_hq(cloud, m, W, H, 1.01)
+    for v in (pcr.PCR_VARIANT_ATOMICMIN, pcr.PCR_VARIANT_DEDUP_EARLYZ):
+        for a, b in zip(r.render_hq(v), hq):
+            assert np.array_equal(a, b), v
+    r.close()
