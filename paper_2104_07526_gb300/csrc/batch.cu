@@ -229,16 +229,17 @@ __global__ void __launch_bounds__(T) k_batch_phase1(const Tables* __restrict__ t
         seen_key[u] = (basic && vis[u]) ? load_relaxed_u64(bv.keys + pix[u]) : 0ull;
         seen_depth[u] = (hq && vis[u]) ? load_relaxed_u32(bv.depth + pix[u]) : 0u;
       }
+      bool group = true;
       if (basic) {
 #pragma unroll
         for (int u = 0; u < U; ++u)
-          emit_key<PCR_VARIANT_EARLYZ>(bv.keys, vis[u], pix[u], make_key(w[u], slot_index<U, kInterleaved>(base, u)), seen_key[u], pol_fb);
+          emit_key<PCR_VARIANT_EARLYZ>(bv.keys, vis[u], pix[u], make_key(w[u], slot_index<U, kInterleaved>(base, u)), seen_key[u], pol_fb, group, u == 0);
       }
       if (hq) {
 #pragma unroll
         for (int u = 0; u < U; ++u)
           emit_depth<PCR_VARIANT_EARLYZ>(bv.depth, vis[u], pix[u], __float_as_uint(w[u]), seen_depth[u],
-                                               pol_fb);
+                                         pol_fb, group, u == 0);
       }
     }
   });

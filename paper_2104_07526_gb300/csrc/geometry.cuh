@@ -125,6 +125,28 @@ __device__ __forceinline__ bool slot_in_range(uint32_t base, int u, uint32_t n, 
   }
 }
 
+// Runs of equal pixels among the neighbouring lanes of a row that are `in`.
+// Called by the whole warp; warp-uniform.
+__device__ __forceinline__ int pixel_runs(bool in, uint32_t pix) {
+  const uint32_t tag = in ? pix : kNoPixel;
+  const uint32_t prev = __shfl_up_sync(kFullMask, tag, 1);
+  return __popc(__ballot_sync(kFullMask, in && (lane_id() == 0 || prev != tag)));
+}
+
+// Whether warp deduplication (Sec. 3.4) pays in a chunk, judged from the
+// lanes of its first row that would write.  With more than kDedupMaxRuns runs
+// the pixels are nearly all distinct (shuffled orders, or fewer points than
+// pixels): the match would find groups of one, and the reductions over a row's
+// groups, whose masks differ from lane to lane, run one group after the other.
+// Without the early test, a shuffled 800M frame took 12.07 ms with the match
+// in every row.  With it, where the test is made only in rows that write at
+// all: a 20k-point frame takes 23.4 us with the match in every row and 11.3
+// with this test, a 50M-point frame in generation order 376 and 301 us; up
+// to 20 runs measure the same, 28 take 14.8 and 313 us, and coherent orders
+// do not change (800M frame 1.853 ms at each).
+constexpr int kDedupMaxRuns = 16;
+__device__ __forceinline__ bool dedup_pays(bool in, uint32_t pix) { return pixel_runs(in, pix) <= kDedupMaxRuns; }
+
 // ---------------------------------------------------------------------------
 // Sec. 3.1-3.4: basic key render
 // ---------------------------------------------------------------------------
@@ -136,10 +158,12 @@ __host__ __device__ constexpr bool reads_early() {
 
 // One point slot after projection: its key (payload P), and `seen`, this
 // lane's earlier read of its pixel (variants with the early test only).
+// `group` carries dedup_pays from a chunk's `first` row to its others; the
+// caller sets it for PCR_VARIANT_DEDUP, the row itself for DEDUP_EARLYZ.
 template <int V, int P = kPayloadIndex>
 __device__ __forceinline__ bool emit_key(unsigned long long* __restrict__ fb, bool vis, uint32_t pix,
                                          unsigned long long key, unsigned long long seen, uint64_t pol,
-                                         bool group = true) {
+                                         bool& group, bool first) {
   if constexpr (V == PCR_VARIANT_ATOMICMIN) {
     // Sec. 3.1: a 64-bit minimum of the key into its pixel's word
     if (vis) red_min_u64(fb + pix, key, pol);
@@ -175,21 +199,30 @@ __device__ __forceinline__ bool emit_key(unsigned long long* __restrict__ fb, bo
     // buffer take part in the deduplication, which the whole warp skips when
     // none is left.  A lane dropped by the early test can never hold a
     // pixel's final minimum, so the set of writers still contains it and the
-    // buffer is the same.
+    // buffer is the same.  The lowest lane of those tied at a group's minimum
+    // depth comes from one vote of the whole row: a second reduction, one
+    // group after the other, made a 100M-point frame in scanline order take
+    // 319 us instead of 292.
     const bool want = vis && key < seen;
     const uint32_t active = __ballot_sync(kFullMask, want);
-    if (active != 0 && want) {
+    if (active == 0u) return false;
+    if (first) group = __popc(active) <= kDedupMaxRuns || dedup_pays(want, pix);
+    if (!group) {
+      if (want) red_min_u64(fb + pix, key, pol);
+      return want;
+    }
+    if (want) {
       const uint32_t peers = __match_any_sync(active, pix);
       const uint32_t hi = key_depth<P>(key);
       const uint32_t hmin = __reduce_min_sync(peers, hi);
-      uint32_t first;
+      uint32_t writer;
       if constexpr (P == kPayloadRgb) {
         const uint32_t tied = __ballot_sync(peers, hi == hmin);
-        first = min_key_lane<P>(tied, hi == hmin, key_payload<P>(key));
+        writer = min_key_lane<P>(tied, hi == hmin, key_payload<P>(key));
       } else {
-        first = __reduce_min_sync(peers, hi == hmin ? lane_id() : 32u);
+        writer = static_cast<uint32_t>(__ffs(__ballot_sync(active, hi == hmin) & peers) - 1);
       }
-      if (lane_id() == first) {
+      if (lane_id() == writer) {
         red_min_u64(fb + pix, key, pol);
         return true;
       }
@@ -229,22 +262,9 @@ __device__ __forceinline__ bool emit_key(unsigned long long* __restrict__ fb, bo
   }
 }
 
-// Whether warp deduplication (Sec. 3.4, without the early test) pays in this
-// chunk, judged from its first row: the runs of equal pixels among
-// neighbouring visible lanes.  With more than kDedupMaxRuns the pixels are
-// nearly all distinct (shuffled orders) and the match would find groups of
-// one.  Warp-uniform.
-constexpr int kDedupMaxRuns = 16;
-__device__ __forceinline__ bool dedup_pays(bool vis0, uint32_t pix0) {
-  const uint32_t tag = vis0 ? pix0 : kNoPixel;
-  const uint32_t prev = __shfl_up_sync(kFullMask, tag, 1);
-  const uint32_t starts = __ballot_sync(kFullMask, vis0 && (lane_id() == 0 || prev != tag));
-  return __popc(starts) <= kDedupMaxRuns;
-}
-
 template <int V>
 __device__ __forceinline__ bool emit_depth(uint32_t* __restrict__ depth, bool vis, uint32_t pix, uint32_t d,
-                                           uint32_t seen, uint64_t pol) {
+                                           uint32_t seen, uint64_t pol, bool& group, bool first) {
   if constexpr (V == PCR_VARIANT_ATOMICMIN) {
     if (vis) red_min_u32(depth + pix, d, pol);
     return vis;
@@ -265,7 +285,13 @@ __device__ __forceinline__ bool emit_depth(uint32_t* __restrict__ depth, bool vi
     static_assert(V == PCR_VARIANT_DEDUP_EARLYZ, "unknown depth variant");
     const bool want = vis && d < seen;
     const uint32_t active = __ballot_sync(kFullMask, want);
-    if (active != 0 && want) {
+    if (active == 0u) return false;
+    if (first) group = __popc(active) <= kDedupMaxRuns || dedup_pays(want, pix);
+    if (!group) {
+      if (want) red_min_u32(depth + pix, d, pol);
+      return want;
+    }
+    if (want) {
       const uint32_t peers = __match_any_sync(active, pix);
       const uint32_t dmin = __reduce_min_sync(peers, d);
       if (lane_id() == static_cast<uint32_t>(__ffs(peers) - 1)) {
@@ -299,6 +325,14 @@ __device__ __forceinline__ uint32_t lanemask_lt() {
   asm("mov.u32 %0, %%lanemask_lt;" : "=r"(m));
   return m;
 }
+
+// In a chunk where fewer than kColorMinJoins lanes share a pixel between
+// their first two points, the lanes' slot-0 runs (four points apart) nearly
+// all lie on different pixels, and the warp step is skipped: 50M points from
+// mid distance take 0.316 ms per HQ frame with 8, 0.322 without the test and
+// 0.334 with 16; from the overview, where it rarely applies, 0.343, 0.342 and
+// 0.352.
+constexpr int kColorMinJoins = 8;
 
 // Colour pass grouping (Listing "hqs_render" adds (r << 32 | g) and
 // (b << 32 | 1) per contributing point; sums do not depend on grouping).
@@ -339,6 +373,7 @@ __device__ __forceinline__ void group_colors(const bool (&contrib)[U], const uin
     }
 #pragma unroll
     for (int u = 1; u < U; ++u) add[u] = contrib[u] && !join[u];
+    if (__popc(__ballot_sync(kFullMask, join[1])) < kColorMinJoins) return;
     // the run from slot 0, over the warp: lanes whose slot 0 does not
     // contribute meet under kNoPixel (never a pixel) and add nothing there
     const uint32_t peers = __match_any_sync(kFullMask, contrib[0] ? pix[0] : kNoPixel);

@@ -103,12 +103,12 @@ __global__ void __launch_bounds__(kThreads, kRenderMinBlocks) k_render_basic(con
       seen[u] = (reads_early<V>() && vis[u]) ? load_relaxed_u64(fb + pix[u]) : 0ull;
       PCR_DEBUG_COUNT(3, reads_early<V>() && vis[u]);
     }
-    const bool group = V != PCR_VARIANT_DEDUP || dedup_pays(vis[0], pix[0]);
+    bool group = V != PCR_VARIANT_DEDUP || dedup_pays(vis[0], pix[0]);
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const bool wrote = emit_key<V, P>(
           fb, vis[u], pix[u], make_payload_key<P>(w[u], P == kPayloadRgb ? r[u].w : slot_index<U, L>(base, u)),
-          seen[u], pol_fb, group);
+          seen[u], pol_fb, group, u == 0);
       PCR_DEBUG_COUNT(0, wrote);
     }
   });
@@ -226,9 +226,10 @@ __global__ void __launch_bounds__(kThreads, kHqMinBlocks) k_hq_depth(const uint4
       seen[u] = (kEarly && vis[u]) ? load_relaxed_u32(depth + pix[u]) : 0u;
       PCR_DEBUG_COUNT(3, kEarly && vis[u]);
     }
+    bool group = true;
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      const bool wrote = emit_depth<V>(depth, vis[u], pix[u], d[u], seen[u], pol_fb);
+      const bool wrote = emit_depth<V>(depth, vis[u], pix[u], d[u], seen[u], pol_fb, group, u == 0);
       PCR_DEBUG_COUNT(1, wrote);
     }
   });
