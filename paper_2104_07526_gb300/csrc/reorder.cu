@@ -6,12 +6,11 @@
 // the high half, both stable, which is a stable sort by the whole code.
 //
 // Radix sort: 8-bit digits, one pass per digit, three steps per pass:
-//   1. k_sort_hist: per tile of 6144 keys (5120 in the random shuffle,
-//      whose passes carry records), count each digit (the first
+//   1. k_sort_hist: per tile of 6144 keys, count each digit (the first
 //      pass's counts come from the kernel that made the keys);
 //   2. exclusive scan of the counts in digit-major order, which gives every
 //      (digit, tile) its first output slot;
-//   3. k_sort_scatter: each warp of a tile takes 768 (640) consecutive keys and
+//   3. k_sort_scatter: each warp of a tile takes 768 consecutive keys and
 //      counts their digits (per 32 keys, one match.any when their digits
 //      form few runs, else eight ballots, one per digit bit);
 //      one prefix over (digit, warp) then gives every warp its first slot
@@ -20,6 +19,8 @@
 //      out run by run, so each digit's keys leave as one contiguous,
 //      coalesced run.
 // Ranks follow index order, so each pass, and the sort, is stable.
+// Random orders (the shuffle, and the order of the 128-point batches) have
+// uniform keys and a sort of their own: random_order.cuh.
 #include <cstdint>
 #include <mutex>
 #include <type_traits>
@@ -56,11 +57,6 @@ constexpr int kSortThreads = 256;
 constexpr int kSortWarps = kSortThreads / 32;
 constexpr int kSortRounds = 24;  // keys per lane in a tile (Morton codes, batch keys)
 constexpr uint32_t kTile = kSortThreads * kSortRounds;
-// The random shuffle's sort carries 16-byte records: tiles of 20 keys per
-// lane keep each block's record window smaller (800M shuffle 34.4 ms with
-// 24, 30.6 with 20, 30.9 with 16).
-constexpr int kShuffleRounds = 20;
-constexpr int kMinRounds = kShuffleRounds < kSortRounds ? kShuffleRounds : kSortRounds;
 template <int ROUNDS>
 constexpr uint32_t kTileOf = kSortThreads * ROUNDS;
 constexpr int kDigitBits = 8;
@@ -78,7 +74,7 @@ constexpr uint32_t kBatch = 128;  // Sec. 4: batches of 128 points
 constexpr int kGatherUnroll = PCR_GATHER_UNROLL;
 
 static_assert(kRadix == kSortThreads, "one digit per thread in the sort kernels");
-static_assert(kSortRounds % 4 == 0 && kShuffleRounds % 4 == 0, "keys per lane read as 16-byte vectors");
+static_assert(kSortRounds % 4 == 0, "keys per lane read as 16-byte vectors");
 
 constexpr uint64_t align_up(uint64_t v) { return (v + 255) & ~uint64_t(255); }
 
@@ -86,7 +82,7 @@ constexpr uint64_t ceil_div(uint64_t a, uint64_t b) { return (a + b - 1) / b; }
 
 // Workspace layout; every region starts on a 256-byte boundary.
 struct Layout {
-  uint64_t pts_copy, keys0, keys1, vals0, vals1, counts, partials, bkeys0, bkeys1, bvals0, bvals1, misc, total;
+  uint64_t pts_copy, keys0, keys1, vals0, vals1, counts, partials, rank, bvals0, bvals1, misc, total;
 };
 
 constexpr uint64_t region(uint64_t& off, uint64_t bytes) {
@@ -97,8 +93,8 @@ constexpr uint64_t region(uint64_t& off, uint64_t bytes) {
 
 constexpr Layout layout(uint64_t n) {
   const uint64_t nb = ceil_div(n, kBatch);
-  const uint64_t tiles = ceil_div(n > nb ? n : nb, kTileOf<kMinRounds>);  // the most any sort has
-  const uint64_t count_words = kRadix * (tiles > 0 ? tiles : 1);
+  const uint64_t tiles = ceil_div(n, kTile);
+  const uint64_t count_words = kRadix * (tiles > 0 ? tiles : 1);  // random orders need fewer (random_counter_words)
   Layout l{};
   uint64_t off = 0;
   l.pts_copy = region(off, 16 * n);
@@ -108,8 +104,7 @@ constexpr Layout layout(uint64_t n) {
   l.vals1 = region(off, 4 * n);
   l.counts = region(off, 4 * count_words);
   l.partials = region(off, 4 * ceil_div(count_words, kScanSeg));
-  l.bkeys0 = region(off, 4 * nb);
-  l.bkeys1 = region(off, 4 * nb);
+  l.rank = region(off, 4 * nb);
   l.bvals0 = region(off, 4 * nb);
   l.bvals1 = region(off, 4 * nb);
   l.misc = region(off, 64);
@@ -369,34 +364,6 @@ __global__ void __launch_bounds__(kSortThreads) k_morton63(const uint4* __restri
   count_tile_digits(sh, valid, counts, tiles);
 }
 
-// SplitMix64 (Steele, Lea and Flood, OOPSLA 2014): output k of the generator
-// seeded with `seed` mixes the state seed + (k + 1) * 0x9E3779B97F4A7C15.
-__device__ __forceinline__ uint64_t splitmix64(uint64_t seed, uint64_t k) {
-  uint64_t z = seed + (k + 1) * 0x9E3779B97F4A7C15ull;
-  z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
-  z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
-  return z ^ (z >> 31);
-}
-
-// Keys for the random orders: the high half of SplitMix64 output i, with the
-// first sort pass's digit counts.
-template <int ROUNDS>
-__global__ void __launch_bounds__(kSortThreads) k_random_keys(uint32_t count, uint64_t seed,
-                                                              uint32_t* __restrict__ keys,
-                                                              uint32_t* __restrict__ counts, uint32_t tiles) {
-  __shared__ TileKeys<ROUNDS> sh;
-  zero_tile_hist(sh);
-  constexpr uint32_t kT = kTileOf<ROUNDS>;
-  const uint64_t tile_base = static_cast<uint64_t>(blockIdx.x) * kT;
-  const uint32_t valid = static_cast<uint32_t>(count - tile_base < kT ? count - tile_base : kT);
-  for (uint32_t j = threadIdx.x; j < valid; j += kSortThreads) {
-    const uint32_t key = static_cast<uint32_t>(splitmix64(seed, tile_base + j) >> 32);
-    keys[tile_base + j] = key;
-    sh.keys[j] = key;
-  }
-  count_tile_digits(sh, valid, counts, tiles);
-}
-
 // --- radix sort ---------------------------------------------------------------
 
 // Lanes of the warp whose 8-bit digit equals this lane's, among the lanes
@@ -477,7 +444,7 @@ __device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t v, uint32_t& t
 // Dynamic shared memory of k_sort_scatter: the tile's keys as loaded, each
 // output slot's input slot, the per-warp first slot of each digit, and per
 // digit the output position minus the tile slot of its first key.  45 KB for
-// 24 keys per lane, 38 KB for 20: four blocks per SM either way.
+// 24 keys per lane: four blocks per SM.
 template <int ROUNDS>
 constexpr size_t scatter_smem() {
   return sizeof(uint32_t) * kTileOf<ROUNDS> + sizeof(uint16_t) * kTileOf<ROUNDS> +
@@ -511,21 +478,16 @@ struct FinalGather {
 // key (the high words of 63-bit codes while their low words are sorted).
 // `vout` may be null when no value is carried; a null `vin` with a `vout`
 // carries each key's input index (the first pass of a sort whose values start
-// as the identity, so they are never written out and read back).  With REC,
-// the 16-byte point record `rin[i]` moves with its key to `rout` (the random
-// order sorts the records themselves: every pass reads them in tile order and
-// writes them in digit runs, instead of one random gather at the end).  With
+// as the identity, so they are never written out and read back).  With
 // `fin.src` the records move as FinalGather says, and `vout` is not written.
-template <bool REC, int ROUNDS>
+template <int ROUNDS>
 __global__ void __launch_bounds__(kSortThreads, 4) k_sort_scatter(const uint32_t* __restrict__ kin,
                                                                   const uint32_t* __restrict__ vin,
                                                                   uint32_t* __restrict__ kout,
                                                                   uint32_t* __restrict__ vout, uint32_t n, int shift,
                                                                   const uint32_t* __restrict__ offsets,
                                                                   uint32_t tiles, const uint32_t* __restrict__ cin,
-                                                                  uint32_t* __restrict__ cout,
-                                                                  const uint4* __restrict__ rin,
-                                                                  uint4* __restrict__ rout, FinalGather fin) {
+                                                                  uint32_t* __restrict__ cout, FinalGather fin) {
   constexpr uint32_t kT = kTileOf<ROUNDS>;  // keys in a tile
   constexpr uint32_t kKeysPerWarp = kT / kSortWarps;
   extern __shared__ __align__(16) uint32_t smem[];
@@ -649,15 +611,10 @@ __global__ void __launch_bounds__(kSortThreads, 4) k_sort_scatter(const uint32_t
         if constexpr (kPerm) fin.perm_out[at] = v;
       }
       if constexpr (kCarried) cout[g] = __ldg(cin + tile_base + src);
-      if constexpr (REC) __stcs(rout + g, __ldg(rin + tile_base + src));
     };
-    // records carried: one key per iteration (unrolled 2, 3, 4 or 8 times the
-    // 800M shuffle took 36.2, 35.9, 38.1 and 39.2 ms against 35.4); records
-    // gathered by index: kGatherUnroll; keys and 4-byte values: eight
-    if constexpr (REC) {
-#pragma unroll 1
-      for (uint32_t l = t; l < total; l += kSortThreads) one(l);
-    } else if constexpr (kGather != 0) {
+    // records gathered by index: kGatherUnroll keys in flight per thread; keys
+    // and 4-byte values: eight
+    if constexpr (kGather != 0) {
 #pragma unroll kGatherUnroll
       for (uint32_t l = t; l < total; l += kSortThreads) one(l);
     } else {
@@ -670,34 +627,27 @@ __global__ void __launch_bounds__(kSortThreads, 4) k_sort_scatter(const uint32_t
   using C2 = std::integral_constant<int, 2>;
   using Yes = std::true_type;
   using No = std::false_type;
-  if constexpr (!REC) {
-    if (fin.src) {
-      auto go = [&](auto values) {
-        if (fin.rank) {
-          if (fin.perm_out) write_out(values, No{}, No{}, C2{}, Yes{});
-          else write_out(values, No{}, No{}, C2{}, No{});
-        } else {
-          if (fin.perm_out) write_out(values, No{}, No{}, C1{}, Yes{});
-          else write_out(values, No{}, No{}, C1{}, No{});
-        }
-      };
-      if (vin) go(C1{});
-      else go(C2{});
-      return;
-    }
+  if (fin.src) {
+    auto go = [&](auto values) {
+      if (fin.rank) {
+        if (fin.perm_out) write_out(values, No{}, No{}, C2{}, Yes{});
+        else write_out(values, No{}, No{}, C2{}, No{});
+      } else {
+        if (fin.perm_out) write_out(values, No{}, No{}, C1{}, Yes{});
+        else write_out(values, No{}, No{}, C1{}, No{});
+      }
+    };
+    if (vin) go(C1{});
+    else go(C2{});
+    return;
   }
   auto go = [&](auto values) {
-    if constexpr (REC) {
-      if (kout) write_out(values, No{}, Yes{}, C0{}, No{});
-      else write_out(values, No{}, No{}, C0{}, No{});
+    if (kout) {
+      if (cout) write_out(values, Yes{}, Yes{}, C0{}, No{});
+      else write_out(values, No{}, Yes{}, C0{}, No{});
     } else {
-      if (kout) {
-        if (cout) write_out(values, Yes{}, Yes{}, C0{}, No{});
-        else write_out(values, No{}, Yes{}, C0{}, No{});
-      } else {
-        if (cout) write_out(values, Yes{}, No{}, C0{}, No{});
-        else write_out(values, No{}, No{}, C0{}, No{});
-      }
+      if (cout) write_out(values, Yes{}, No{}, C0{}, No{});
+      else write_out(values, No{}, No{}, C0{}, No{});
     }
   };
   if (!vout) go(C0{});
@@ -833,24 +783,21 @@ cudaError_t exclusive_scan(uint32_t* a, uint64_t len, uint32_t* partials, cudaSt
 // words; the last pass writes no keys.  With `carry` (may be null), a second
 // value per key moves with it through its own two buffers, and with
 // `carry_last` (may be null) the last pass writes the carried words there
-// instead.  With `recs` (may be null), a 16-byte record moves with each key.
-// vals may hold null buffers when no value is needed.  With `index_values`
+// instead.  vals may hold null buffers when no value is needed.  With `index_values`
 // the values start as each key's index: the first pass makes them, and
 // vals[0] is never read.  With `first_counted` the kernel that made the keys
-// has already written the first pass's digit counts (k_morton, k_morton63,
-// k_random_keys).  With `fin` (may be null) the last pass moves the records
+// has already written the first pass's digit counts (k_morton, k_morton63).  With `fin` (may be null) the last pass moves the records
 // as FinalGather says, instead of writing the values.
 template <int ROUNDS>
 cudaError_t radix_sort(uint32_t* keys[2], uint32_t* vals[2], uint32_t count, int key_bits, uint32_t* counts,
                        uint32_t* partials, cudaStream_t s, int& out, bool index_values, bool first_counted,
                        uint32_t* const* carry = nullptr, uint32_t* carry_last = nullptr,
-                       uint4* const* recs = nullptr, const FinalGather* fin = nullptr) {
+                       const FinalGather* fin = nullptr) {
   out = 0;
   if (count == 0) return cudaSuccess;
   constexpr size_t kSmem = scatter_smem<ROUNDS>();
   const uint32_t tiles = static_cast<uint32_t>(ceil_div(count, kTileOf<ROUNDS>));
-  cudaError_t e = cudaFuncSetAttribute(recs ? k_sort_scatter<true, ROUNDS> : k_sort_scatter<false, ROUNDS>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kSmem));
+  cudaError_t e = cudaFuncSetAttribute(k_sort_scatter<ROUNDS>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kSmem));
   if (e != cudaSuccess) return e;
   for (int shift = 0; shift < key_bits; shift += kDigitBits) {
     const bool last = shift + kDigitBits >= key_bits;
@@ -860,14 +807,9 @@ cudaError_t radix_sort(uint32_t* keys[2], uint32_t* vals[2], uint32_t count, int
     const uint32_t* vin = (index_values && shift == 0) ? nullptr : vals[out];
     uint32_t* kout = last ? nullptr : keys[out ^ 1];
     const FinalGather f = (last && fin) ? *fin : FinalGather{};
-    if (recs)
-      k_sort_scatter<true, ROUNDS><<<tiles, kSortThreads, kSmem, s>>>(
-          keys[out], vin, kout, vals[out ^ 1], count, shift, counts, tiles, nullptr, nullptr, recs[out],
-          recs[out ^ 1], f);
-    else
-      k_sort_scatter<false, ROUNDS><<<tiles, kSortThreads, kSmem, s>>>(
-          keys[out], vin, kout, vals[out ^ 1], count, shift, counts, tiles, carry ? carry[out] : nullptr,
-          carry ? (last && carry_last ? carry_last : carry[out ^ 1]) : nullptr, nullptr, nullptr, f);
+    k_sort_scatter<ROUNDS><<<tiles, kSortThreads, kSmem, s>>>(
+        keys[out], vin, kout, vals[out ^ 1], count, shift, counts, tiles, carry ? carry[out] : nullptr,
+        carry ? (last && carry_last ? carry_last : carry[out ^ 1]) : nullptr, f);
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     out ^= 1;
@@ -875,15 +817,15 @@ cudaError_t radix_sort(uint32_t* keys[2], uint32_t* vals[2], uint32_t count, int
   return cudaSuccess;
 }
 
-// --- shuffled Morton: batch slots; record copy -------------------------------------
+}  // namespace
+}  // namespace pcr
 
-// Slot of each batch in the sorted batch order: rank[order[t]] = t.
-__global__ void k_batch_rank(const uint32_t* __restrict__ order, uint32_t nb, uint32_t* __restrict__ rank) {
-  for (uint64_t t = blockIdx.x * 256ull + threadIdx.x; t < nb; t += gridDim.x * 256ull) {
-    const uint32_t b = order[t];
-    if (debug_in_range(b, nb)) rank[b] = static_cast<uint32_t>(t);
-  }
-}
+#include "random_order.cuh"
+
+namespace pcr {
+namespace {
+
+// --- record copy -------------------------------------------------------------------
 
 __global__ void __launch_bounds__(256) k_copy16(const uint4* __restrict__ src, uint4* __restrict__ dst, uint32_t n) {
   for (uint64_t i = blockIdx.x * 256ull + threadIdx.x; i < n; i += gridDim.x * 256ull) dst[i] = __ldcs(src + i);
@@ -951,18 +893,9 @@ cudaError_t launch_reorder(uint4* pts, uint32_t n, uint64_t seed, int mode, void
   cudaError_t e = cudaSuccess;
   int out = 0;
   if (mode == PCR_ORDER_SHUFFLE) {
-    // the records themselves are sorted by their random keys (4 passes, an
-    // even number: they end back in the caller's buffer); indices ride along
-    // only when the permutation is asked for, with the caller's buffer as
-    // the value buffer the last pass writes
-    const uint32_t stiles = static_cast<uint32_t>(ceil_div(n, kTileOf<kShuffleRounds>));
-    k_random_keys<kShuffleRounds><<<stiles, kSortThreads, 0, s>>>(n, seed, keys[0], counts, stiles);
-    uint32_t* ivals[2] = {perm_out, perm_out ? vals[1] : nullptr};
-    uint4* recs[2] = {pts, copy};
-    e = radix_sort<kShuffleRounds>(keys, ivals, n, 32, counts, partials, s, out, true, true, nullptr, nullptr, recs);
-    if (e != cudaSuccess) return e;
-    if (out != 0) return cudaErrorUnknown;  // 32-bit keys take 4 passes: the values end in ivals[0]
-    return cudaSuccess;
+    RandomOut to;
+    to.perm = perm_out;
+    return random_order<true>(pts, copy, n, seed, vals, counts, partials, to, s, d);
   }
   // The sort's last pass moves the records from their copy to their final
   // positions: the sorted positions, or with the batch shuffle, the slots of
@@ -973,23 +906,19 @@ cudaError_t launch_reorder(uint4* pts, uint32_t n, uint64_t seed, int mode, void
   fin.perm_out = perm_out;
   if (mode == PCR_ORDER_MORTON_SHUFFLE128 || mode == PCR_ORDER_MORTON63_SHUFFLE128) {
     const uint32_t nb = static_cast<uint32_t>(ceil_div(n, kBatch));
-    uint32_t* bkeys[2] = {reinterpret_cast<uint32_t*>(ws + l.bkeys0), reinterpret_cast<uint32_t*>(ws + l.bkeys1)};
     uint32_t* bvals[2] = {reinterpret_cast<uint32_t*>(ws + l.bvals0), reinterpret_cast<uint32_t*>(ws + l.bvals1)};
-    const uint32_t btiles = static_cast<uint32_t>(ceil_div(nb, kTile));
-    k_random_keys<kSortRounds><<<btiles, kSortThreads, 0, s>>>(nb, seed, bkeys[0], counts, btiles);
-    int bout = 0;
-    e = radix_sort<kSortRounds>(bkeys, bvals, nb, 32, counts, partials, s, bout, true, true);
+    RandomOut to;
+    to.rank = reinterpret_cast<uint32_t*>(ws + l.rank);
+    e = random_order<false>(nullptr, nullptr, nb, seed, bvals, counts, partials, to, s, d);
     if (e != cudaSuccess) return e;
-    k_batch_rank<<<stream_grid(nb, d), 256, 0, s>>>(bvals[bout], nb, bkeys[0]);
-    fin.rank = bkeys[0];
+    fin.rank = to.rank;
     fin.nb = nb;
   }
   k_bounds_init<<<1, 32, 0, s>>>(misc);
   if (mode == PCR_ORDER_MORTON || mode == PCR_ORDER_MORTON_SHUFFLE128) {
     k_bounds<<<grid, 256, 0, s>>>(pts, n, misc, copy);
     k_morton<<<tiles, kSortThreads, 0, s>>>(pts, n, misc, keys[0], counts, tiles);
-    e = radix_sort<kSortRounds>(keys, vals, n, 30, counts, partials, s, out, true, true, nullptr, nullptr, nullptr,
-                                &fin);
+    e = radix_sort<kSortRounds>(keys, vals, n, 30, counts, partials, s, out, true, true, nullptr, nullptr, &fin);
     if (e != cudaSuccess) return e;
     return cudaGetLastError();
   }
@@ -1007,8 +936,7 @@ cudaError_t launch_reorder(uint4* pts, uint32_t n, uint64_t seed, int mode, void
   if (e != cudaSuccess) return e;
   if (a != 0) return cudaErrorUnknown;  // 4 passes: the values are in vals[0]
   k_copy16<<<grid, 256, 0, s>>>(pts, copy, n);
-  e = radix_sort<kSortRounds>(keys, vals, n, 31, counts, partials, s, out, false, false, nullptr, nullptr, nullptr,
-                              &fin);
+  e = radix_sort<kSortRounds>(keys, vals, n, 31, counts, partials, s, out, false, false, nullptr, nullptr, &fin);
   if (e != cudaSuccess) return e;
   return cudaGetLastError();
 }

@@ -241,3 +241,18 @@ def test_debug_reorder_and_batch_match_the_oracle_with_silent_checks(debug_lib, 
                     assert np.array_equal(b["hq_rg"].cpu().numpy().view(np.uint64), rg), config
                     assert np.array_equal(b["hq_ba"].cpu().numpy().view(np.uint64), ba), config
         assert pcr.pcr_last_device_error(c.handle) == 0
+
+
+def test_debug_shuffle_with_buckets_past_shared_memory(debug_lib, oracle):
+    """Debug builds sort every other bucket of the random order the way a
+    bucket too large for shared memory is sorted: with one partition pass
+    (records from the workspace's copy) and with two (in place, by way of it)."""
+    from gpu_helpers import reorder_gpu
+    with pcr.Context(0, stream=torch.cuda.current_stream()) as c:
+        for n in (9_001, 4_100_001):
+            cloud = torch.arange(4 * n, dtype=torch.int32).reshape(n, 4)
+            expect = oracle.reorder(cloud.numpy(), n, pcr.PCR_ORDER_SHUFFLE).astype(np.int64)
+            dev = cloud.cuda()
+            assert np.array_equal(reorder_gpu(c.handle, dev, n, pcr.PCR_ORDER_SHUFFLE), expect), n
+            assert torch.equal(dev.cpu(), cloud[torch.from_numpy(expect)]), n
+        assert pcr.pcr_last_device_error(c.handle) == 0

@@ -127,3 +127,19 @@ def test_reorder_errors(r):
     with pytest.raises(pcr.PcrError) as e:
         pcr.pcr_reorder_morton_shuffle128(r.h, dev.data_ptr() + 4, n, 0, 0, ws)
     assert e.value.status == pcr.PCR_ERR_ARG
+
+
+@pytest.mark.parametrize("n", [1983, 1984, 1985, 4095, 4096, 4097, 20_011, 2048 * 1984, 2048 * 1984 + 1])
+def test_shuffle_at_its_pass_limits(r, oracle, n):
+    """The random order's buckets hold 1984 records on average: one bucket and
+    two, tiles of 4096 and one more, the most records one partition pass
+    splits and the first size that takes two."""
+    cloud = torch.arange(4 * n, dtype=torch.int32).reshape(n, 4)
+    expect = oracle.reorder(cloud.numpy(), 11 * n, pcr.PCR_ORDER_SHUFFLE).astype(np.int64)
+    dev = cloud.cuda()
+    assert np.array_equal(reorder_gpu(r.h, dev, 11 * n, pcr.PCR_ORDER_SHUFFLE), expect)
+    assert torch.equal(dev.cpu(), cloud[torch.from_numpy(expect)])
+    ws = torch.empty(pcr.pcr_reorder_workspace_size(n), dtype=torch.uint8, device="cuda")
+    dev = cloud.cuda()
+    pcr.pcr_reorder_morton_shuffle128(r.h, dev, n, 11 * n, pcr.PCR_ORDER_SHUFFLE, ws)
+    assert torch.equal(dev.cpu(), cloud[torch.from_numpy(expect)])
