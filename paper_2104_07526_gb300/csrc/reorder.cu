@@ -80,6 +80,24 @@ constexpr uint64_t align_up(uint64_t v) { return (v + 255) & ~uint64_t(255); }
 
 constexpr uint64_t ceil_div(uint64_t a, uint64_t b) { return (a + b - 1) / b; }
 
+// Small clouds.  Their sorts are bound by launches and by blocks too few to
+// fill the GPU, so a pass is one launch of smaller tiles: every scatter block
+// sums the counts of the tiles before its own, and counts the next pass's
+// digits as it writes (one global atomic per key).  Morton order, one launch
+// per pass against five on tiles of 6144: 60k points 136 -> 51 us, 130k
+// 149 -> 62, 390k 150 -> 81, 780k 174 -> 111, 1.5M 221 -> 170, 2.2M
+// 254 -> 240; shuffled Morton of 100k 253 -> 66 us (bound by the chain of
+// launches: seven, of about 6 us each).  Past the last limit the sums over
+// tiles cost more than a scan (3.1M: 345 against 300 us with 512 tiles); 12
+// keys per lane take over from 4 where their sums are shorter (190k points:
+// 70 against 75 us).  Keys per lane of a small sort's tiles; 0: not small.
+constexpr int small_rounds(uint64_t n) {
+  return n <= 128 * kTileOf<4> ? 4 : n <= 256 * kTileOf<12> ? 12 : n <= 384 * kTileOf<24> ? 24 : 0;
+}
+constexpr uint32_t kSumUnroll = 32;   // counts of other tiles in flight per thread (16: 74 us, 32: 66 at 100k)
+constexpr uint32_t kBoundsParts = 128;  // blocks of a small cloud's k_bounds, at most
+constexpr int kBoundsValues = 6;  // per block of a small cloud's k_bounds
+
 // Workspace layout; every region starts on a 256-byte boundary.
 struct Layout {
   uint64_t pts_copy, keys0, keys1, vals0, vals1, counts, partials, rank, bvals0, bvals1, misc, total;
@@ -141,7 +159,9 @@ static_assert(kSortRounds % kMortonUnroll == 0, "whole rounds of records per til
 // Per axis min and max over non-NaN coordinates.  -0 is folded into +0 (the
 // codes do not depend on the sign of a zero bound).  With `copy`, the records
 // are also copied there (the source the sort's last pass moves them from),
-// saving a pass.
+// saving a pass.  SMALL: block b writes its own bounds to misc[6 b .. 6 b + 5]
+// (k_morton joins them) instead of joining them in misc[0 .. 5].
+template <bool SMALL>
 __global__ void __launch_bounds__(256) k_bounds(const uint4* __restrict__ pts, uint32_t n, uint32_t* misc,
                                                 uint4* __restrict__ copy) {
   uint32_t lo[3] = {0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu};
@@ -175,6 +195,25 @@ __global__ void __launch_bounds__(256) k_bounds(const uint4* __restrict__ pts, u
   for (int a = 0; a < 3; ++a) {
     lo[a] = __reduce_min_sync(kFullMask, lo[a]);
     hi[a] = __reduce_max_sync(kFullMask, hi[a]);
+  }
+  if constexpr (SMALL) {
+    __shared__ uint32_t s_bounds[8][kBoundsValues];
+    if (lane_id() == 0) {
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        // no value: the identities k_bounds_init starts from
+        s_bounds[threadIdx.x >> 5][a] = min(lo[a], 0xFF800000u);
+        s_bounds[threadIdx.x >> 5][3 + a] = max(hi[a], 0x007FFFFFu);
+      }
+    }
+    __syncthreads();
+    if (threadIdx.x < kBoundsValues) {
+      uint32_t v = s_bounds[0][threadIdx.x];
+      for (int w = 1; w < 8; ++w)
+        v = threadIdx.x < 3 ? min(v, s_bounds[w][threadIdx.x]) : max(v, s_bounds[w][threadIdx.x]);
+      misc[kBoundsValues * blockIdx.x + threadIdx.x] = v;
+    }
+    return;
   }
   if (lane_id() == 0) {
 #pragma unroll
@@ -217,7 +256,18 @@ struct alignas(16) TileKeys {
   uint32_t hist[kSortWarps][kRadix];
 };
 
-template <int ROUNDS>
+// Counts of later passes of a small sort: a kernel with one block per tile
+// clears the tile's row of each (null: none).
+struct ClearRows {
+  uint32_t* at[3] = {nullptr, nullptr, nullptr};
+};
+__device__ __forceinline__ void clear_rows(const ClearRows& rows) {
+#pragma unroll
+  for (int k = 0; k < 3; ++k)
+    if (rows.at[k]) rows.at[k][blockIdx.x * kRadix + threadIdx.x] = 0u;
+}
+
+template <int ROUNDS, bool SMALL>
 __device__ __forceinline__ void count_tile_digits(TileKeys<ROUNDS>& sh, uint32_t valid, uint32_t* __restrict__ counts,
                                                   uint32_t tiles) {
   __syncthreads();  // the tile's keys are in place
@@ -258,6 +308,10 @@ __device__ __forceinline__ void count_tile_digits(TileKeys<ROUNDS>& sh, uint32_t
   uint32_t c = 0;
 #pragma unroll
   for (int w = 0; w < kSortWarps; ++w) c += sh.hist[w][threadIdx.x];
+  if constexpr (SMALL) {
+    if (counts) counts[blockIdx.x * kRadix + threadIdx.x] = c;
+    return;
+  }
   counts[static_cast<uint64_t>(threadIdx.x) * tiles + blockIdx.x] = c;
 }
 
@@ -268,48 +322,84 @@ __device__ __forceinline__ void zero_tile_hist(TileKeys<ROUNDS>& sh) {
 }
 
 
-// Sec. 5: Morton code over the cube with the bounds' minimum corner and the
-// largest extent as side, 10 levels.
+// The root cube: the bounds' minimum corner, and the cells per unit of length
+// along its side (`cells` over the largest extent; 0 for a degenerate cube,
+// whose codes are all 0).  misc holds `parts` sets of bounds, or one.
+template <bool SMALL>
+struct RootCube {
+  float lo[3];
+  float scale;
+  bool degenerate;
+
+  __device__ __forceinline__ RootCube(const uint32_t* __restrict__ misc, uint32_t parts, float cells) {
+    uint32_t b[kBoundsValues];
+    if constexpr (SMALL) {
+      __shared__ uint32_t s_bounds[kBoundsValues];
+      const uint32_t k = threadIdx.x >> 5;
+      if (k < kBoundsValues) {
+        uint32_t v = misc[k];
+        for (uint32_t p = lane_id(); p < parts; p += 32) {
+          const uint32_t o = misc[kBoundsValues * p + k];
+          v = k < 3 ? min(v, o) : max(v, o);
+        }
+        v = k < 3 ? __reduce_min_sync(kFullMask, v) : __reduce_max_sync(kFullMask, v);
+        if (lane_id() == 0) s_bounds[k] = v;
+      }
+      __syncthreads();
+      for (int a = 0; a < kBoundsValues; ++a) b[a] = s_bounds[a];
+    } else {
+      for (int a = 0; a < kBoundsValues; ++a) b[a] = misc[a];
+    }
+    float ext = 0.0f;
+    for (int a = 0; a < 3; ++a) {
+      lo[a] = order_float(b[a]);
+      const float e = __fsub_rn(order_float(b[3 + a]), lo[a]);
+      if (a == 0 || e > ext) ext = e;
+    }
+    degenerate = !(ext > 0.0f) || !(ext < __int_as_float(kInfBits));
+    scale = degenerate ? 0.0f : __fdiv_rn(cells, ext);
+  }
+};
+
+// Sec. 5: Morton code over the root cube, 10 levels.  `parts`: see RootCube.
+// SMALL: the counts go tile by tile (null: a single tile's sort needs none).
+template <int ROUNDS, bool SMALL>
 __global__ void __launch_bounds__(kSortThreads) k_morton(const uint4* __restrict__ pts, uint32_t n,
                                                          const uint32_t* __restrict__ misc,
                                                          uint32_t* __restrict__ keys, uint32_t* __restrict__ counts,
-                                                         uint32_t tiles) {
-  __shared__ TileKeys<kSortRounds> sh;
+                                                         uint32_t tiles, uint32_t parts,
+                                                         ClearRows zero) {
+  __shared__ TileKeys<ROUNDS> sh;
+  constexpr uint32_t kT = kTileOf<ROUNDS>;
   zero_tile_hist(sh);
-  const float lo[3] = {order_float(misc[0]), order_float(misc[1]), order_float(misc[2])};
-  const float hi[3] = {order_float(misc[3]), order_float(misc[4]), order_float(misc[5])};
-  float ext = __fsub_rn(hi[0], lo[0]);
-  const float ey = __fsub_rn(hi[1], lo[1]);
-  const float ez = __fsub_rn(hi[2], lo[2]);
-  if (ey > ext) ext = ey;
-  if (ez > ext) ext = ez;
-  const bool degenerate = !(ext > 0.0f) || !(ext < __int_as_float(kInfBits));
-  const float scale = degenerate ? 0.0f : __fdiv_rn(1024.0f, ext);
-  const uint64_t tile_base = static_cast<uint64_t>(blockIdx.x) * kTile;
-  const uint32_t valid = static_cast<uint32_t>(n - tile_base < kTile ? n - tile_base : kTile);
-  // kMortonUnroll records per thread in flight at a time
-  for (uint32_t j0 = threadIdx.x; j0 < valid; j0 += kSortThreads * kMortonUnroll) {
-    uint4 r[kMortonUnroll];
+  if constexpr (SMALL) clear_rows(zero);
+  const RootCube<SMALL> cube(misc, parts, 1024.0f);
+  const uint64_t tile_base = static_cast<uint64_t>(blockIdx.x) * kT;
+  const uint32_t valid = static_cast<uint32_t>(n - tile_base < kT ? n - tile_base : kT);
+  // kUnroll records per thread in flight at a time
+  constexpr int kUnroll = ROUNDS < kMortonUnroll ? ROUNDS : kMortonUnroll;
+  for (uint32_t j0 = threadIdx.x; j0 < valid; j0 += kSortThreads * kUnroll) {
+    uint4 r[kUnroll];
 #pragma unroll
-    for (int u = 0; u < kMortonUnroll; ++u) {
+    for (int u = 0; u < kUnroll; ++u) {
       const uint32_t j = j0 + kSortThreads * u;
-      r[u] = (!degenerate && j < valid) ? __ldcs(pts + tile_base + j) : make_uint4(0u, 0u, 0u, 0u);
+      r[u] = (!cube.degenerate && j < valid) ? __ldcs(pts + tile_base + j) : make_uint4(0u, 0u, 0u, 0u);
     }
 #pragma unroll
-    for (int u = 0; u < kMortonUnroll; ++u) {
+    for (int u = 0; u < kUnroll; ++u) {
       const uint32_t j = j0 + kSortThreads * u;
       if (j >= valid) break;
       uint32_t code = 0;
-      if (!degenerate) {
-        code = (spread3(quantise(__uint_as_float(r[u].x), lo[0], scale)) << 2) |
-               (spread3(quantise(__uint_as_float(r[u].y), lo[1], scale)) << 1) |
-               spread3(quantise(__uint_as_float(r[u].z), lo[2], scale));
+      if (!cube.degenerate) {
+        code = (spread3(quantise(__uint_as_float(r[u].x), cube.lo[0], cube.scale)) << 2) |
+               (spread3(quantise(__uint_as_float(r[u].y), cube.lo[1], cube.scale)) << 1) |
+               spread3(quantise(__uint_as_float(r[u].z), cube.lo[2], cube.scale));
       }
       keys[tile_base + j] = code;
       sh.keys[j] = code;
     }
   }
-  count_tile_digits(sh, valid, counts, tiles);
+  count_tile_digits<ROUNDS, SMALL>(sh, valid, counts, tiles);
 }
 
 // Spread the low 21 bits of v so bit i lands on bit 3i.
@@ -332,36 +422,32 @@ __device__ __forceinline__ uint32_t quantise21(float v, float lo, float scale) {
 
 // Sec. 5 with the paper's 21 levels: the same cube, 2^21 cells per axis.
 // Writes the code's low 32 bits to keys_lo and its high 31 bits to hi.
+template <int ROUNDS, bool SMALL>
 __global__ void __launch_bounds__(kSortThreads) k_morton63(const uint4* __restrict__ pts, uint32_t n,
                                                            const uint32_t* __restrict__ misc,
                                                            uint32_t* __restrict__ keys_lo, uint32_t* __restrict__ hi,
-                                                           uint32_t* __restrict__ counts, uint32_t tiles) {
-  __shared__ TileKeys<kSortRounds> sh;
+                                                           uint32_t* __restrict__ counts, uint32_t tiles, uint32_t parts,
+                                                           ClearRows zero) {
+  __shared__ TileKeys<ROUNDS> sh;
+  constexpr uint32_t kT = kTileOf<ROUNDS>;
   zero_tile_hist(sh);
-  const float lo[3] = {order_float(misc[0]), order_float(misc[1]), order_float(misc[2])};
-  const float top[3] = {order_float(misc[3]), order_float(misc[4]), order_float(misc[5])};
-  float ext = __fsub_rn(top[0], lo[0]);
-  const float ey = __fsub_rn(top[1], lo[1]);
-  const float ez = __fsub_rn(top[2], lo[2]);
-  if (ey > ext) ext = ey;
-  if (ez > ext) ext = ez;
-  const bool degenerate = !(ext > 0.0f) || !(ext < __int_as_float(kInfBits));
-  const float scale = degenerate ? 0.0f : __fdiv_rn(2097152.0f, ext);
-  const uint64_t tile_base = static_cast<uint64_t>(blockIdx.x) * kTile;
-  const uint32_t valid = static_cast<uint32_t>(n - tile_base < kTile ? n - tile_base : kTile);
+  if constexpr (SMALL) clear_rows(zero);
+  const RootCube<SMALL> cube(misc, parts, 2097152.0f);
+  const uint64_t tile_base = static_cast<uint64_t>(blockIdx.x) * kT;
+  const uint32_t valid = static_cast<uint32_t>(n - tile_base < kT ? n - tile_base : kT);
   for (uint32_t j = threadIdx.x; j < valid; j += kSortThreads) {
     uint64_t code = 0;
-    if (!degenerate) {
+    if (!cube.degenerate) {
       const uint4 r = __ldcs(pts + tile_base + j);
-      code = (spread3_21(quantise21(__uint_as_float(r.x), lo[0], scale)) << 2) |
-             (spread3_21(quantise21(__uint_as_float(r.y), lo[1], scale)) << 1) |
-             spread3_21(quantise21(__uint_as_float(r.z), lo[2], scale));
+      code = (spread3_21(quantise21(__uint_as_float(r.x), cube.lo[0], cube.scale)) << 2) |
+             (spread3_21(quantise21(__uint_as_float(r.y), cube.lo[1], cube.scale)) << 1) |
+             spread3_21(quantise21(__uint_as_float(r.z), cube.lo[2], cube.scale));
     }
     keys_lo[tile_base + j] = static_cast<uint32_t>(code);
     hi[tile_base + j] = static_cast<uint32_t>(code >> 32);
     sh.keys[j] = static_cast<uint32_t>(code);
   }
-  count_tile_digits(sh, valid, counts, tiles);
+  count_tile_digits<ROUNDS, SMALL>(sh, valid, counts, tiles);
 }
 
 // --- radix sort ---------------------------------------------------------------
@@ -393,9 +479,12 @@ __device__ __forceinline__ uint32_t digit_peers(uint32_t d, uint32_t valid) {
 // the lower digits) have long runs, which one add per key would turn into
 // many same-address shared-memory atomics.  The eight warps' counters are
 // summed at the end.
-template <int ROUNDS>
+// SMALL: the counts go tile by tile.
+template <int ROUNDS, bool SMALL>
 __global__ void __launch_bounds__(kSortThreads) k_sort_hist(const uint32_t* __restrict__ keys, uint32_t n, int shift,
-                                                            uint32_t* __restrict__ counts, uint32_t tiles) {
+                                                            uint32_t* __restrict__ counts, uint32_t tiles,
+                                                            ClearRows zero) {
+  if constexpr (SMALL) clear_rows(zero);
   __shared__ uint32_t hist[kSortWarps][kRadix];
 #pragma unroll
   for (int w = 0; w < kSortWarps; ++w) hist[w][threadIdx.x] = 0;
@@ -434,7 +523,8 @@ __global__ void __launch_bounds__(kSortThreads) k_sort_hist(const uint32_t* __re
   uint32_t c = 0;
 #pragma unroll
   for (int w = 0; w < kSortWarps; ++w) c += hist[w][threadIdx.x];
-  counts[static_cast<uint64_t>(threadIdx.x) * tiles + blockIdx.x] = c;
+  if constexpr (SMALL) counts[blockIdx.x * kRadix + threadIdx.x] = c;
+  else counts[static_cast<uint64_t>(threadIdx.x) * tiles + blockIdx.x] = c;
 }
 
 template <int NT>
@@ -473,6 +563,14 @@ struct FinalGather {
   uint32_t nb = 0;                 // batches (with rank)
 };
 
+// A small sort's pass (SMALL): its counts lie tile by tile in `offsets`, not
+// scanned (null for a single tile), and it adds the next pass's counts to
+// `next` (may be null), by the digit at next_shift of the keys it writes.
+struct SmallPass {
+  uint32_t* next = nullptr;
+  int next_shift = 0;
+};
+
 // `kout` may be null: the last pass of a sort writes no keys (nothing reads
 // them).  `cin`/`cout` (may be null): a second 32-bit value carried with each
 // key (the high words of 63-bit codes while their low words are sorted).
@@ -480,14 +578,15 @@ struct FinalGather {
 // carries each key's input index (the first pass of a sort whose values start
 // as the identity, so they are never written out and read back).  With
 // `fin.src` the records move as FinalGather says, and `vout` is not written.
-template <int ROUNDS>
+template <int ROUNDS, bool SMALL>
 __global__ void __launch_bounds__(kSortThreads, 4) k_sort_scatter(const uint32_t* __restrict__ kin,
                                                                   const uint32_t* __restrict__ vin,
                                                                   uint32_t* __restrict__ kout,
                                                                   uint32_t* __restrict__ vout, uint32_t n, int shift,
                                                                   const uint32_t* __restrict__ offsets,
                                                                   uint32_t tiles, const uint32_t* __restrict__ cin,
-                                                                  uint32_t* __restrict__ cout, FinalGather fin) {
+                                                                  uint32_t* __restrict__ cout, FinalGather fin,
+                                                                  SmallPass small) {
   constexpr uint32_t kT = kTileOf<ROUNDS>;  // keys in a tile
   constexpr uint32_t kKeysPerWarp = kT / kSortWarps;
   extern __shared__ __align__(16) uint32_t smem[];
@@ -507,7 +606,24 @@ __global__ void __launch_bounds__(kSortThreads, 4) k_sort_scatter(const uint32_t
   asm volatile("cp.async.commit_group;" ::: "memory");
 #pragma unroll
   for (int w = 0; w < kSortWarps; ++w) wbase[w * kRadix + t] = 0;
-  const uint32_t global_start = offsets[static_cast<uint64_t>(t) * tiles + blockIdx.x];
+  // output position of the tile's first key with digit t
+  uint32_t global_start = 0;
+  if (SMALL && offsets) {
+    uint32_t before = 0, all = 0, total;
+    for (uint32_t o0 = 0; o0 < tiles; o0 += kSumUnroll) {
+      uint32_t c[kSumUnroll];
+#pragma unroll
+      for (uint32_t u = 0; u < kSumUnroll; ++u) c[u] = o0 + u < tiles ? __ldg(offsets + (o0 + u) * kRadix + t) : 0u;
+#pragma unroll
+      for (uint32_t u = 0; u < kSumUnroll; ++u) {
+        all += c[u];
+        before += o0 + u < blockIdx.x ? c[u] : 0u;
+      }
+    }
+    global_start = block_exclusive_scan<kSortThreads>(all, total) + before;
+  } else if constexpr (!SMALL) {
+    global_start = offsets[static_cast<uint64_t>(t) * tiles + blockIdx.x];
+  }
   asm volatile("cp.async.wait_all;" ::: "memory");
   __syncthreads();
   // this warp's 768 consecutive keys; pass 1 counts their digits, and each
@@ -548,7 +664,7 @@ __global__ void __launch_bounds__(kSortThreads, 4) k_sort_scatter(const uint32_t
   }
   uint32_t total;
   const uint32_t start = block_exclusive_scan<kSortThreads>(run, total);
-  delta[t] = global_start - start;  // modulo 2^32: output position = delta + tile slot
+  delta[t] = !SMALL || offsets ? global_start - start : 0u;  // modulo 2^32: output position = delta + tile slot
 #pragma unroll
   for (int w = 0; w < kSortWarps; ++w) wbase[w * kRadix + t] += start;
   __syncthreads();
@@ -611,6 +727,9 @@ __global__ void __launch_bounds__(kSortThreads, 4) k_sort_scatter(const uint32_t
         if constexpr (kPerm) fin.perm_out[at] = v;
       }
       if constexpr (kCarried) cout[g] = __ldg(cin + tile_base + src);
+      if constexpr (SMALL && kKeys) {
+        if (small.next) atomicAdd(small.next + g / kT * kRadix + ((key >> small.next_shift) & (kRadix - 1)), 1u);
+      }
     };
     // records gathered by index: kGatherUnroll keys in flight per thread; keys
     // and 4-byte values: eight
@@ -797,24 +916,55 @@ cudaError_t radix_sort(uint32_t* keys[2], uint32_t* vals[2], uint32_t count, int
   if (count == 0) return cudaSuccess;
   constexpr size_t kSmem = scatter_smem<ROUNDS>();
   const uint32_t tiles = static_cast<uint32_t>(ceil_div(count, kTileOf<ROUNDS>));
-  cudaError_t e = cudaFuncSetAttribute(k_sort_scatter<ROUNDS>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kSmem));
+  cudaError_t e = cudaFuncSetAttribute(k_sort_scatter<ROUNDS, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kSmem));
   if (e != cudaSuccess) return e;
   for (int shift = 0; shift < key_bits; shift += kDigitBits) {
     const bool last = shift + kDigitBits >= key_bits;
-    if (!(first_counted && shift == 0)) k_sort_hist<ROUNDS><<<tiles, kSortThreads, 0, s>>>(keys[out], count, shift, counts, tiles);
+    if (!(first_counted && shift == 0)) k_sort_hist<ROUNDS, false><<<tiles, kSortThreads, 0, s>>>(keys[out], count, shift, counts, tiles, ClearRows{});
     e = exclusive_scan(counts, static_cast<uint64_t>(kRadix) * tiles, partials, s);
     if (e != cudaSuccess) return e;
     const uint32_t* vin = (index_values && shift == 0) ? nullptr : vals[out];
     uint32_t* kout = last ? nullptr : keys[out ^ 1];
     const FinalGather f = (last && fin) ? *fin : FinalGather{};
-    k_sort_scatter<ROUNDS><<<tiles, kSortThreads, kSmem, s>>>(
+    k_sort_scatter<ROUNDS, false><<<tiles, kSortThreads, kSmem, s>>>(
         keys[out], vin, kout, vals[out ^ 1], count, shift, counts, tiles, carry ? carry[out] : nullptr,
-        carry ? (last && carry_last ? carry_last : carry[out ^ 1]) : nullptr, f);
+        carry ? (last && carry_last ? carry_last : carry[out ^ 1]) : nullptr, f, SmallPass{});
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     out ^= 1;
   }
   return cudaSuccess;
+}
+
+// Four passes of a small sort (key_bits of 25 to 32), one launch each.
+// counts[p] (null for a single tile) holds or receives pass p's counts: the
+// first ones are made, the next two clear; `last_counts` says that the last
+// ones are too, otherwise k_sort_hist makes them.
+template <int ROUNDS>
+cudaError_t small_sort(uint32_t* const keys[2], uint32_t* const vals[2], uint32_t count, bool index_values,
+                       uint32_t* const counts[4], bool last_counts, uint32_t* const* carry, uint32_t* carry_last,
+                       const FinalGather& fin, cudaStream_t s) {
+  constexpr int kPasses = 4;
+  const uint32_t tiles = static_cast<uint32_t>(ceil_div(count, kTileOf<ROUNDS>));
+  constexpr size_t kSmem = scatter_smem<ROUNDS>();
+  cudaError_t e = cudaFuncSetAttribute(k_sort_scatter<ROUNDS, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       static_cast<int>(kSmem));
+  if (e != cudaSuccess) return e;
+  for (int p = 0; p < kPasses; ++p) {
+    const int from = p & 1, to = from ^ 1;
+    const bool last = p == kPasses - 1;
+    SmallPass pass;
+    if (p + 1 < kPasses - (last_counts ? 0 : 1)) pass.next = counts[p + 1];
+    pass.next_shift = (p + 1) * kDigitBits;
+    if (last && !last_counts && counts[p])
+      k_sort_hist<ROUNDS, true><<<tiles, kSortThreads, 0, s>>>(keys[from], count, p * kDigitBits, counts[p], tiles,
+                                                               ClearRows{});
+    k_sort_scatter<ROUNDS, true><<<tiles, kSortThreads, kSmem, s>>>(
+        keys[from], index_values && p == 0 ? nullptr : vals[from], last ? nullptr : keys[to], vals[to], count,
+        p * kDigitBits, counts[p], tiles, carry ? carry[from] : nullptr,
+        carry ? (last ? carry_last : carry[to]) : nullptr, last ? fin : FinalGather{}, pass);
+  }
+  return cudaGetLastError();
 }
 
 }  // namespace
@@ -877,6 +1027,52 @@ void forget_noalloc_scratch(int device) {
 
 uint64_t reorder_workspace_bytes(uint64_t n) { return layout(n).total; }
 
+namespace {
+
+// Morton orders of a small cloud: bounds, codes and one launch per sort pass.
+// The counts of its passes lie in buffers that are free while they are needed:
+//   30-bit: pass 0 in vals[0]; passes 1 and 2 in the points (read from their
+//     copy from the codes on), pass 3 in keys[0];
+//   63-bit: pass 0 in vals[0], 1 to 3 behind the high halves in the copy
+//     region, 4 to 6 in the points (copied by then), 7 in keys[0].
+// A tile of 1024 keys or more has 1 KB of counts, so a set takes at most 2 n
+// bytes (n with a full last tile): two fit a 4-byte buffer, and three fit
+// behind two of them in the copy's 16 n.  A single tile has no counts.
+template <int ROUNDS>
+cudaError_t small_morton(uint4* pts, uint32_t n, bool fine, uint4* copy, uint32_t* const keys[2],
+                         uint32_t* const vals[2], uint32_t* const hi[2], uint32_t* bounds, const FinalGather& fin,
+                         unsigned grid, cudaStream_t s) {
+  const uint32_t tiles = static_cast<uint32_t>(ceil_div(n, kTileOf<ROUNDS>));
+  const uint64_t words = static_cast<uint64_t>(kRadix) * tiles;
+  auto counts_at = [&](void* base, int k) {
+    return tiles > 1 ? static_cast<uint32_t*>(base) + k * words : nullptr;
+  };
+  const uint32_t steps = static_cast<uint32_t>(ceil_div(n, 256 * kStreamUnroll));
+  const uint32_t parts = steps < kBoundsParts ? steps : kBoundsParts;
+  k_bounds<true><<<parts, 256, 0, s>>>(pts, n, bounds, fine ? nullptr : copy);
+  if (!fine) {
+    uint32_t* const counts[4] = {counts_at(vals[0], 0), counts_at(pts, 0), counts_at(pts, 1), counts_at(keys[0], 0)};
+    k_morton<ROUNDS, true><<<tiles, kSortThreads, 0, s>>>(copy, n, bounds, keys[0], counts[0], tiles, parts,
+                                                         ClearRows{{counts[1], counts[2], nullptr}});
+    return small_sort<ROUNDS>(keys, vals, n, true, counts, false, nullptr, nullptr, fin, s);
+  }
+  uint32_t* const free_words = hi[1] + (hi[1] - hi[0]);
+  uint32_t* const low[4] = {counts_at(vals[0], 0), counts_at(free_words, 0), counts_at(free_words, 1),
+                            counts_at(free_words, 2)};
+  k_morton63<ROUNDS, true><<<tiles, kSortThreads, 0, s>>>(pts, n, bounds, keys[0], hi[0], low[0], tiles, parts,
+                                                         ClearRows{{low[1], low[2], low[3]}});
+  const cudaError_t e = small_sort<ROUNDS>(keys, vals, n, true, low, true, hi, keys[0], FinalGather{}, s);
+  if (e != cudaSuccess) return e;
+  k_copy16<<<grid, 256, 0, s>>>(pts, copy, n);
+  uint32_t* const high[4] = {counts_at(pts, 0), counts_at(pts, 1), counts_at(pts, 2), counts_at(keys[0], 0)};
+  if (high[0])
+    k_sort_hist<ROUNDS, true><<<tiles, kSortThreads, 0, s>>>(keys[0], n, 0, high[0], tiles,
+                                                             ClearRows{{high[1], high[2], nullptr}});
+  return small_sort<ROUNDS>(keys, vals, n, false, high, false, nullptr, nullptr, fin, s);
+}
+
+}  // namespace
+
 cudaError_t launch_reorder(uint4* pts, uint32_t n, uint64_t seed, int mode, void* workspace, uint32_t* perm_out,
                            cudaStream_t s, const Device& d) {
   if (n == 0) return cudaSuccess;
@@ -914,10 +1110,20 @@ cudaError_t launch_reorder(uint4* pts, uint32_t n, uint64_t seed, int mode, void
     fin.rank = to.rank;
     fin.nb = nb;
   }
+  const bool fine = mode == PCR_ORDER_MORTON63 || mode == PCR_ORDER_MORTON63_SHUFFLE128;
+  // 63-bit codes: buffers of their high halves in the record-copy region
+  uint32_t* hi[2] = {reinterpret_cast<uint32_t*>(ws + l.pts_copy),
+                     reinterpret_cast<uint32_t*>(ws + l.pts_copy) + align_up(4ull * n) / 4};
+  switch (small_rounds(n)) {
+    case 4: return small_morton<4>(pts, n, fine, copy, keys, vals, hi, counts, fin, grid, s);
+    case 12: return small_morton<12>(pts, n, fine, copy, keys, vals, hi, counts, fin, grid, s);
+    case 24: return small_morton<24>(pts, n, fine, copy, keys, vals, hi, counts, fin, grid, s);
+    default: break;
+  }
   k_bounds_init<<<1, 32, 0, s>>>(misc);
-  if (mode == PCR_ORDER_MORTON || mode == PCR_ORDER_MORTON_SHUFFLE128) {
-    k_bounds<<<grid, 256, 0, s>>>(pts, n, misc, copy);
-    k_morton<<<tiles, kSortThreads, 0, s>>>(pts, n, misc, keys[0], counts, tiles);
+  if (!fine) {
+    k_bounds<false><<<grid, 256, 0, s>>>(pts, n, misc, copy);
+    k_morton<kSortRounds, false><<<tiles, kSortThreads, 0, s>>>(pts, n, misc, keys[0], counts, tiles, 1, ClearRows{});
     e = radix_sort<kSortRounds>(keys, vals, n, 30, counts, partials, s, out, true, true, nullptr, nullptr, &fin);
     if (e != cudaSuccess) return e;
     return cudaGetLastError();
@@ -927,10 +1133,8 @@ cudaError_t launch_reorder(uint4* pts, uint32_t n, uint64_t seed, int mode, void
   // pass leaves them in keys[0] (the low halves are no longer needed), which
   // frees the region for the record copy.  Then the high halves are sorted,
   // and that sort's last pass moves the records.
-  uint32_t* hi[2] = {reinterpret_cast<uint32_t*>(ws + l.pts_copy),
-                     reinterpret_cast<uint32_t*>(ws + l.pts_copy) + align_up(4ull * n) / 4};
-  k_bounds<<<grid, 256, 0, s>>>(pts, n, misc, nullptr);
-  k_morton63<<<tiles, kSortThreads, 0, s>>>(pts, n, misc, keys[0], hi[0], counts, tiles);
+  k_bounds<false><<<grid, 256, 0, s>>>(pts, n, misc, nullptr);
+  k_morton63<kSortRounds, false><<<tiles, kSortThreads, 0, s>>>(pts, n, misc, keys[0], hi[0], counts, tiles, 1, ClearRows{});
   int a = 0;
   e = radix_sort<kSortRounds>(keys, vals, n, 32, counts, partials, s, a, true, true, hi, keys[0]);
   if (e != cudaSuccess) return e;

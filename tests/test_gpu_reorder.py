@@ -143,3 +143,37 @@ def test_shuffle_at_its_pass_limits(r, oracle, n):
     dev = cloud.cuda()
     pcr.pcr_reorder_morton_shuffle128(r.h, dev, n, 11 * n, pcr.PCR_ORDER_SHUFFLE, ws)
     assert torch.equal(dev.cpu(), cloud[torch.from_numpy(expect)])
+
+
+@pytest.mark.parametrize("n", [255, 1023, 1024, 1025, 2049, 128 * 1024, 128 * 1024 + 1, 256 * 3072, 256 * 3072 + 1,
+                               384 * 6144, 384 * 6144 + 1])
+def test_reorder_at_the_limits_of_small_sorts(r, oracle, n):
+    """One tile and two, the last size of each tile size, and the first that
+    takes the three-kernel passes; half of the points lie on few cells."""
+    rng = np.random.default_rng(n)
+    cloud = scenes.random_cloud(n, seed=n).numpy()
+    dense = rng.random(n) < 0.5
+    cloud[dense, :3] = rng.uniform(-0.01, 0.01, (int(dense.sum()), 3)).astype(np.float32).view(np.int32)
+    for mode in (pcr.PCR_ORDER_MORTON, pcr.PCR_ORDER_MORTON63, pcr.PCR_ORDER_MORTON_SHUFFLE128):
+        expect = oracle.reorder(cloud, 5 + n, mode)
+        dev = torch.from_numpy(cloud.copy()).cuda()
+        assert np.array_equal(reorder_gpu(r.h, dev, 5 + n, mode), expect), mode
+        assert np.array_equal(dev.cpu().numpy(), oracle.gather(cloud, expect)), mode
+
+
+def test_small_reorder_of_points_without_bounds(r, oracle):
+    """Every coordinate NaN, one axis NaN, infinities: the bounds' joins."""
+    base = scenes.random_cloud(3001, seed=1).numpy()
+    for spoil in ("all", "axis", "inf"):
+        cloud = base.copy()
+        if spoil == "all":
+            cloud[:, :3] = np.float32(np.nan).view(np.int32)
+        elif spoil == "axis":
+            cloud[:, 1] = np.float32(np.nan).view(np.int32)
+        else:
+            cloud[::7, 0] = np.float32(np.inf).view(np.int32)
+            cloud[3::7, 2] = np.float32(-np.inf).view(np.int32)
+        for mode in MODES:
+            expect = oracle.reorder(cloud, 3, mode)
+            dev = torch.from_numpy(cloud.copy()).cuda()
+            assert np.array_equal(reorder_gpu(r.h, dev, 3, mode), expect), (spoil, mode)
