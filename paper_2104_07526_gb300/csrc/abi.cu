@@ -472,8 +472,8 @@ pcr_status pcr_render_hq(pcr_ctx* ctx, float depth_factor, int variant, int clea
   if (clear) e = pcr::launch_clear_hq(ctx->depth, ctx->rg, ctx->ba, pixels(ctx), ctx->stream, ctx->dev);
   if (e == cudaSuccess) e = pcr::launch_hq_depth(variant, ctx->points, n, v, ctx->depth, ctx->stream, ctx->dev);
   if (e == cudaSuccess)
-    e = pcr::launch_hq_color(variant, ctx->points, n, v, depth_factor, ctx->depth, ctx->rg, ctx->ba, ctx->stream,
-                             ctx->dev);
+    e = pcr::launch_hq_color(variant, ctx->points, n, v, depth_factor, ctx->depth, sizeof(uint32_t), ctx->rg, ctx->ba,
+                             ctx->stream, ctx->dev);
   return from_cuda(e);
 }
 

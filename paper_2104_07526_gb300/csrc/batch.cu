@@ -3,10 +3,11 @@
 // as one CUDA graph.
 //
 // Each pass over a cloud's points projects every point for a group of that
-// cloud's views.  Phase 1 (index 0 in the tables) writes the basic key (Sec.
-// 3.1-3.2, with the early depth test) and the high-quality depth (Sec. 3.5)
-// from one projection; phase 2 (index 1), after all depth buffers are
-// complete, adds the high-quality colours (summed inside the warp first).  A
+// cloud's views.  Phase 1 (index 0 in the tables) writes each view's basic keys
+// (Sec. 3.1-3.2, with the early depth test), whose upper words are the
+// high-quality depths too, or the depths (Sec. 3.5) of a view without basic
+// frame; phase 2 (index 1), after all depths are complete, adds the
+// high-quality colours (summed inside the warp first).  A
 // group holds as many views as fit an L2 budget (framebuffer bytes the pass
 // touches), packed first-fit by decreasing size, so the atomics and early
 // depth reads of a pass stay in L2 while the point stream passes through; a
@@ -191,6 +192,12 @@ __device__ __forceinline__ void for_each_batch_chunk(const Shared& sh, int phase
   }
 }
 
+// The depths of a view's pixels after phase 1.
+__host__ __device__ __forceinline__ DepthSource depth_source(const BatchView& v) {
+  if (v.flags & PCR_BATCH_BASIC) return {reinterpret_cast<const uint32_t*>(v.keys) + 1, sizeof(unsigned long long)};
+  return {v.depth, sizeof(uint32_t)};
+}
+
 template <int U>
 __device__ __forceinline__ void project_all(const ViewParams& vp, const uint4 (&r)[U], const bool (&ok)[U],
                                             uint32_t (&pix)[U], float (&w)[U], bool (&vis)[U]) {
@@ -202,44 +209,45 @@ __device__ __forceinline__ void project_all(const ViewParams& vp, const uint4 (&
   debug_check_view_pixels<U>(vp, pix, vis);
 }
 
-// Phase 1: per view of the pass, basic key and HQ depth, each with the
-// early depth test (on GB300 the fastest exact form once the buffer is
-// filling: warp deduplication saves no atomics after the early test), both
-// from one projection.
+// Phase 1: per view of the pass, basic keys, or depths for a view that asks
+// for the high-quality frame alone: where both are asked for, the keys' upper
+// words are the depths (phase 2 reads them there, and the resolve writes the
+// depth buffer).  Early depth test without deduplication: the passes were
+// bound by the L1 (83% busy) with 1.5 atomics per point and view when both
+// buffers were kept, and the match costs more than the atomics it saves (8
+// clouds x 8 views, keys and colours: 22.2 ms with both buffers, 19.7 with the
+// keys alone, 20.6 with deduplication).
 template <int U, int T>
 __global__ void __launch_bounds__(T) k_batch_phase1(const Tables* __restrict__ tables) {
   const Shared sh = load_tables(tables, 0);
   const uint64_t pol_stream = policy_evict_first();
   const uint64_t pol_fb = policy_evict_last();
-  for_each_batch_chunk<U, kInterleaved>(sh, 0, pol_stream, [&](const BatchGroup& grp, const uint4(&r)[U], uint32_t base,
-                                                 const bool(&ok)[U]) {
+  constexpr int L = kInterleaved;
+  for_each_batch_chunk<U, L>(sh, 0, pol_stream, [&](const BatchGroup& grp, const uint4(&r)[U], uint32_t base,
+                                                    const bool(&ok)[U]) {
     for (uint32_t i = grp.first; i < grp.first + grp.count; ++i) {
       const BatchView& bv = sh.views[sh.order[i]];
       uint32_t pix[U];
       float w[U];
       bool vis[U];
       project_all<U>(bv.vp, r, ok, pix, w, vis);
-      // both early reads of every slot first: one L2 round trip per view
-      const bool basic = bv.flags & PCR_BATCH_BASIC;
-      const bool hq = bv.flags & PCR_BATCH_HQ;
-      unsigned long long seen_key[U];
-      uint32_t seen_depth[U];
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        seen_key[u] = (basic && vis[u]) ? load_relaxed_u64(bv.keys + pix[u]) : 0ull;
-        seen_depth[u] = (hq && vis[u]) ? load_relaxed_u32(bv.depth + pix[u]) : 0u;
-      }
+      // every slot's early read first: one L2 round trip per view
       bool group = true;
-      if (basic) {
+      if (bv.flags & PCR_BATCH_BASIC) {
+        unsigned long long seen[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) seen[u] = vis[u] ? load_relaxed_u64(bv.keys + pix[u]) : 0ull;
 #pragma unroll
         for (int u = 0; u < U; ++u)
-          emit_key<PCR_VARIANT_EARLYZ>(bv.keys, vis[u], pix[u], make_key(w[u], slot_index<U, kInterleaved>(base, u)), seen_key[u], pol_fb, group, u == 0);
-      }
-      if (hq) {
+          emit_key<PCR_VARIANT_EARLYZ>(bv.keys, vis[u], pix[u], make_key(w[u], slot_index<U, L>(base, u)), seen[u], pol_fb, group,
+                           u == 0);
+      } else {
+        uint32_t seen[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) seen[u] = vis[u] ? load_relaxed_u32(bv.depth + pix[u]) : 0u;
 #pragma unroll
         for (int u = 0; u < U; ++u)
-          emit_depth<PCR_VARIANT_EARLYZ>(bv.depth, vis[u], pix[u], __float_as_uint(w[u]), seen_depth[u],
-                                         pol_fb, group, u == 0);
+          emit_depth<PCR_VARIANT_EARLYZ>(bv.depth, vis[u], pix[u], __float_as_uint(w[u]), seen[u], pol_fb, group, u == 0);
       }
     }
   });
@@ -262,81 +270,118 @@ __global__ void __launch_bounds__(T, 1024 / T) k_batch_phase2(const Tables* __re
       bool vis[U];
       project_all<U>(bv.vp, r, ok, pix, w, vis);
       bool contrib[U];
-      contributes<U>(bv.depth, factor, pix, w, vis, contrib);
+      contributes<U>(depth_source(bv), factor, pix, w, vis, contrib);
       emit_colors<U, true>(bv.rg, bv.ba, contrib, pix, r, pol_fb);
     }
   });
 }
 
-// Clear and resolve walk the pixels of all views as one sequence.  The view
-// of a pixel is found by one search per warp (lane 0's pixel); lanes whose
-// pixel lies past that view's end search on their own.
-__device__ __forceinline__ uint32_t view_of_pixel(const Shared& sh, uint64_t p) {
-  const uint64_t p0 = __shfl_sync(kFullMask, p, 0);
-  uint32_t vi = 0;
-  if (lane_id() == 0)
-    vi = last_not_above(sh.hdr.num_views, p0, [&](uint32_t i) { return sh.views[i].first_pixel; });
-  vi = __shfl_sync(kFullMask, vi, 0);
-  const uint64_t end = vi + 1 < sh.hdr.num_views ? sh.views[vi + 1].first_pixel : sh.hdr.total_pixels;
-  if (p >= end) vi = last_not_above(sh.hdr.num_views, p, [&](uint32_t i) { return sh.views[i].first_pixel; });
-  return vi;
+// Clear and resolve walk the views' pixels in tiles of kScreenTile: one search
+// per block and tile finds the view, and a thread takes four neighbouring
+// pixels at a time, as 16-byte vectors where the view's buffers allow (the
+// interface promises each buffer's element size).  f(bv, q, count): `count`
+// pixels from pixel q of the view, four or, at a view's end, fewer.  108M
+// pixels with both frames clear in 0.46 ms and resolve in 0.93 (one pixel per
+// thread and a search per warp: 0.56 and 0.99); both are bound by memory, the
+// resolve by its colour gathers too.
+constexpr uint64_t kScreenTile = 4096;
+template <class F>
+__device__ __forceinline__ void for_each_pixel_group(const Shared& sh, F&& f) {
+  for (uint64_t tile = blockIdx.x; tile < sh.hdr.total_tiles; tile += gridDim.x) {
+    const uint32_t vi =
+        last_not_above(sh.hdr.num_views, tile, [&](uint32_t i) { return sh.views[i].first_tile; });
+    const BatchView& bv = sh.views[vi];
+    const uint64_t npx = static_cast<uint64_t>(bv.vp.width) * bv.vp.height;
+    const uint64_t first = (tile - bv.first_tile) * kScreenTile;
+    const uint64_t end = first + kScreenTile < npx ? first + kScreenTile : npx;
+    for (uint64_t q = first + 4 * threadIdx.x; q < end; q += 4 * kThreads)
+      f(bv, q, end - q < 4 ? static_cast<int>(end - q) : 4);
+  }
+}
+
+__device__ __forceinline__ bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
+
+// Four words, or `count` of them, from and to a buffer.
+__device__ __forceinline__ void store_words(uint32_t* p, const uint32_t (&v)[4], int count) {
+  if (count == 4 && aligned16(p)) {
+    *reinterpret_cast<uint4*>(p) = make_uint4(v[0], v[1], v[2], v[3]);
+  } else {
+    for (int k = 0; k < 4; ++k)
+      if (k < count) p[k] = v[k];
+  }
+}
+__device__ __forceinline__ void fill_words(unsigned long long* p, unsigned long long v, int count) {
+  if (count == 4 && aligned16(p)) {
+    ulonglong2* q = reinterpret_cast<ulonglong2*>(p);
+    q[0] = q[1] = make_ulonglong2(v, v);
+  } else {
+    for (int k = 0; k < 4; ++k)
+      if (k < count) p[k] = v;
+  }
+}
+__device__ __forceinline__ void load_words(const unsigned long long* p, unsigned long long (&v)[4], int count) {
+  if (count == 4 && aligned16(p)) {
+    const ulonglong2* q = reinterpret_cast<const ulonglong2*>(p);
+    const ulonglong2 a = q[0], b = q[1];
+    v[0] = a.x, v[1] = a.y, v[2] = b.x, v[3] = b.y;
+  } else {
+    for (int k = 0; k < 4; ++k) v[k] = k < count ? p[k] : 0ull;
+  }
 }
 
 __global__ void __launch_bounds__(kThreads) k_batch_clear(const Tables* __restrict__ tables) {
   const Shared sh = load_tables(tables, -1);
-  const BatchHeader& hdr = sh.hdr;
-  const BatchView* views = sh.views;
-  const uint64_t stride = static_cast<uint64_t>(gridDim.x) * blockDim.x;
-  const uint64_t rounds = (hdr.total_pixels + stride - 1) / stride;  // every lane runs the same rounds
-  for (uint64_t k = 0; k < rounds; ++k) {
-    const uint64_t p = k * stride + blockIdx.x * static_cast<uint64_t>(blockDim.x) + threadIdx.x;
-    const uint32_t vi = view_of_pixel(sh, p < hdr.total_pixels ? p : hdr.total_pixels - 1);
-    if (p >= hdr.total_pixels) continue;
-    const BatchView& bv = views[vi];
-    const uint64_t q = p - bv.first_pixel;
-    if (bv.flags & PCR_BATCH_BASIC) bv.keys[q] = kEmptyKey;
+  for_each_pixel_group(sh, [&](const BatchView& bv, uint64_t q, int count) {
+    if (bv.flags & PCR_BATCH_BASIC) fill_words(bv.keys + q, kEmptyKey, count);
     if (bv.flags & PCR_BATCH_HQ) {
-      bv.depth[q] = kInfBits;
-      bv.rg[q] = 0ull;
-      bv.ba[q] = 0ull;
+      if (!(bv.flags & PCR_BATCH_BASIC)) store_words(bv.depth + q, {kInfBits, kInfBits, kInfBits, kInfBits}, count);
+      fill_words(bv.rg + q, 0ull, count);
+      fill_words(bv.ba + q, 0ull, count);
     }
-  }
+  });
 }
 
+// Images, and the depth buffers of views whose depths are their keys' (see
+// k_batch_phase1).
 __global__ void __launch_bounds__(kThreads) k_batch_resolve(const Tables* __restrict__ tables) {
   const Shared sh = load_tables(tables, -1);
-  const BatchHeader& hdr = sh.hdr;
-  const BatchView* views = sh.views;
-  const BatchCloud* clouds = sh.clouds;
-  const uint32_t background = hdr.background;
-  const uint64_t stride = static_cast<uint64_t>(gridDim.x) * blockDim.x;
-  const uint64_t rounds = (hdr.total_pixels + stride - 1) / stride;  // every lane runs the same rounds
-  for (uint64_t k = 0; k < rounds; ++k) {
-    const uint64_t p = k * stride + blockIdx.x * static_cast<uint64_t>(blockDim.x) + threadIdx.x;
-    const uint32_t vi = view_of_pixel(sh, p < hdr.total_pixels ? p : hdr.total_pixels - 1);
-    if (p >= hdr.total_pixels) continue;
-    const BatchView& bv = views[vi];
-    const uint64_t q = p - bv.first_pixel;
-    if ((bv.flags & PCR_BATCH_BASIC) && bv.image) {
-      const unsigned long long k = bv.keys[q];
-      const uint32_t idx = static_cast<uint32_t>(k);
-      const BatchCloud& cl = clouds[bv.cloud];
-      uint32_t c = background;
-      if (k != kEmptyKey && idx < cl.n) c = __ldg(reinterpret_cast<const uint32_t*>(cl.pts) + 4ull * idx + 3);
-      bv.image[q] = c;
-    }
-    if ((bv.flags & PCR_BATCH_HQ) && bv.hq_image) {
-      const unsigned long long s_rg = bv.rg[q];
-      const unsigned long long s_ba = bv.ba[q];
-      const uint32_t a = static_cast<uint32_t>(s_ba);
-      uint32_t c = background;
-      if (a != 0) {
-        c = min(static_cast<uint32_t>(s_rg >> 32) / a, 255u) | (min(static_cast<uint32_t>(s_rg) / a, 255u) << 8) |
-            (min(static_cast<uint32_t>(s_ba >> 32) / a, 255u) << 16) | 0xFF000000u;
+  const uint32_t background = sh.hdr.background;
+  for_each_pixel_group(sh, [&](const BatchView& bv, uint64_t q, int count) {
+    const bool hq = bv.flags & PCR_BATCH_HQ;
+    if ((bv.flags & PCR_BATCH_BASIC) && (bv.image || hq)) {
+      unsigned long long key[4];
+      load_words(bv.keys + q, key, count);
+      if (bv.image) {
+        const BatchCloud& cl = sh.clouds[bv.cloud];
+        uint32_t c[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const uint32_t idx = static_cast<uint32_t>(key[k]);
+          c[k] = background;
+          if (key[k] != kEmptyKey && idx < cl.n && k < count)
+            c[k] = __ldg(reinterpret_cast<const uint32_t*>(cl.pts) + 4ull * idx + 3);
+        }
+        store_words(bv.image + q, c, count);
       }
-      bv.hq_image[q] = c;
+      if (hq) {
+        uint32_t d[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) d[k] = key[k] == kEmptyKey ? kInfBits : static_cast<uint32_t>(key[k] >> 32);
+        store_words(bv.depth + q, d, count);
+      }
     }
-  }
+    if (hq && bv.hq_image) {
+      unsigned long long rg[4], ba[4];
+      load_words(bv.rg + q, rg, count);
+      load_words(bv.ba + q, ba, count);
+      uint32_t c[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        c[k] = average_color(static_cast<uint32_t>(rg[k] >> 32), static_cast<uint32_t>(rg[k]),
+                             static_cast<uint32_t>(ba[k] >> 32), static_cast<uint32_t>(ba[k]), background);
+      store_words(bv.hq_image + q, c, count);
+    }
+  });
 }
 
 // Launch configurations the autotuner chooses among: threads per block, and
@@ -393,7 +438,9 @@ cudaError_t launch_single(const Tables& h, uint32_t vi, int phase, cudaStream_t 
     if (e == cudaSuccess && (v.flags & PCR_BATCH_HQ))
       e = launch_hq_depth(PCR_VARIANT_DEDUP_EARLYZ, c.pts, c.n, v.vp, v.depth, s, d);
   } else if (v.flags & PCR_BATCH_HQ) {
-    e = launch_hq_color(PCR_VARIANT_DEDUP_EARLYZ, c.pts, c.n, v.vp, h.hdr.depth_factor, v.depth, v.rg, v.ba, s, d);
+    const DepthSource depth = depth_source(v);
+    e = launch_hq_color(PCR_VARIANT_DEDUP_EARLYZ, c.pts, c.n, v.vp, h.hdr.depth_factor, depth.base, depth.step, v.rg, v.ba,
+                        s, d);
   }
   return e;
 }
@@ -431,8 +478,9 @@ void build_groups(Tables* t, const pcr_batch_cloud* clouds, uint32_t num_clouds,
       if (v.cloud != c) continue;
       const uint64_t px = static_cast<uint64_t>(v.width) * static_cast<uint64_t>(v.height);
       uint64_t bytes = 0;
-      if (phase == 0) bytes = px * (((v.flags & PCR_BATCH_BASIC) ? 8u : 0u) + ((v.flags & PCR_BATCH_HQ) ? 4u : 0u));
-      else if (v.flags & PCR_BATCH_HQ) bytes = px * 20u;  // depth read, two 64-bit sums
+      const uint32_t depth_bytes = (v.flags & PCR_BATCH_BASIC) ? 8u : 4u;  // in the keys, or on their own
+      if (phase == 0) bytes = px * depth_bytes;
+      else if (v.flags & PCR_BATCH_HQ) bytes = px * (16u + depth_bytes);  // two 64-bit sums, depth read
       if (bytes > 0) mine.emplace_back(bytes, i);
     }
     std::stable_sort(mine.begin(), mine.end(), [](const auto& a, const auto& b) { return a.first > b.first; });
@@ -485,7 +533,7 @@ void batch_build_tables(const pcr_batch_cloud* clouds, uint32_t num_clouds, cons
     t->clouds[c].pts = static_cast<const uint4*>(clouds[c].points);
     t->clouds[c].n = static_cast<uint32_t>(clouds[c].n);
   }
-  uint64_t pixel = 0;
+  uint64_t tile = 0;
   uint32_t hq = 0;
   for (uint32_t j = 0; j < num_views; ++j) {
     const pcr_batch_view& in = views[j];
@@ -507,11 +555,11 @@ void batch_build_tables(const pcr_batch_cloud* clouds, uint32_t num_clouds, cons
     bv.rg = static_cast<unsigned long long*>(in.hq_rg);
     bv.ba = static_cast<unsigned long long*>(in.hq_ba);
     bv.hq_image = static_cast<uint32_t*>(in.hq_image);
-    bv.first_pixel = pixel;
-    pixel += static_cast<uint64_t>(in.width) * static_cast<uint64_t>(in.height);
+    bv.first_tile = tile;
+    tile += (static_cast<uint64_t>(in.width) * static_cast<uint64_t>(in.height) + kScreenTile - 1) / kScreenTile;
     if (in.flags & PCR_BATCH_HQ) ++hq;
   }
-  t->hdr.total_pixels = pixel;
+  t->hdr.total_tiles = tile;
   t->hdr.hq_views = hq;
   build_groups(t, clouds, num_clouds, views, num_views, 0, l2_budget);
   build_groups(t, clouds, num_clouds, views, num_views, 1, l2_budget);

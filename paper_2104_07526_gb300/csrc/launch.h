@@ -30,9 +30,11 @@ cudaError_t launch_render_basic(int variant, const uint4* pts, uint32_t n, const
                                 unsigned long long* keys, cudaStream_t s, const Device& d);
 cudaError_t launch_hq_depth(int variant, const uint4* pts, uint32_t n, const ViewParams& v, uint32_t* depth,
                             cudaStream_t s, const Device& d);
+// depth_base, depth_step: the pixels' depths and the bytes between them (4 for
+// a depth buffer, 8 for the upper words of a key buffer).
 cudaError_t launch_hq_color(int variant, const uint4* pts, uint32_t n, const ViewParams& v, float depth_factor,
-                            const uint32_t* depth, unsigned long long* rg, unsigned long long* ba, cudaStream_t s,
-                            const Device& d);
+                            const uint32_t* depth_base, uint32_t depth_step, unsigned long long* rg,
+                            unsigned long long* ba, cudaStream_t s, const Device& d);
 cudaError_t launch_resolve_basic(const unsigned long long* keys, uint64_t npx, const uint4* pts, uint32_t n,
                                  uint32_t background, uint32_t* out, cudaStream_t s, const Device& d);
 cudaError_t launch_hq1r_color(int variant, const uint4* pts, uint32_t n, const ViewParams& v, float depth_factor,
@@ -67,7 +69,7 @@ constexpr uint32_t kBatchMaxViews = PCR_BATCH_MAX_VIEWS;
 struct BatchHeader {
   uint32_t num_clouds;
   uint32_t num_views;
-  uint64_t total_pixels;  // sum of view sizes
+  uint64_t total_tiles;  // screen tiles of all views
   uint32_t hq_views;
   uint32_t background;
   float depth_factor;
@@ -103,7 +105,7 @@ struct BatchView {
   unsigned long long* rg;
   unsigned long long* ba;
   uint32_t* hq_image;
-  uint64_t first_pixel;  // offset of this view in the concatenated pixels
+  uint64_t first_tile;  // offset of this view in the concatenated screen tiles
 };
 
 uint64_t batch_workspace_bytes();

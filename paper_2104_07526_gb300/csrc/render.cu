@@ -238,7 +238,7 @@ __global__ void __launch_bounds__(kThreads, kHqMinBlocks) k_hq_depth(const uint4
 // Colour pass (Listing "hqs_render"): see group_colors.
 template <bool AGG, int U, bool V8>
 __global__ void __launch_bounds__(kThreads, kHqMinBlocks) k_hq_color(const uint4* __restrict__ pts, uint32_t n, ViewParams v,
-                                                       float factor, const uint32_t* __restrict__ depth,
+                                                       float factor, DepthSource depth,
                                                        unsigned long long* __restrict__ rg,
                                                        unsigned long long* __restrict__ ba) {
   const uint64_t pol_stream = policy_evict_first();
@@ -336,7 +336,7 @@ __device__ __forceinline__ void hq1r_settle(unsigned long long* __restrict__ pri
 template <bool AGG, int U, bool V8>
 __global__ void __launch_bounds__(kThreads, PCR_HQ1R_MIN_BLOCKS)
     k_hq1r_color(const uint4* __restrict__ pts, uint32_t n, ViewParams v, float factor,
-                 const uint32_t* __restrict__ depth, unsigned long long* __restrict__ primary,
+                 DepthSource depth, unsigned long long* __restrict__ primary,
                  unsigned long long* __restrict__ rg, unsigned long long* __restrict__ ba) {
   const uint64_t pol_stream = policy_evict_first();
   const uint64_t pol_fb = policy_evict_last();
@@ -454,15 +454,8 @@ __global__ void k_resolve_hq(const unsigned long long* __restrict__ rg, const un
        p += static_cast<uint64_t>(gridDim.x) * blockDim.x) {
     const unsigned long long s_rg = rg[p];
     const unsigned long long s_ba = ba[p];
-    const uint32_t a = static_cast<uint32_t>(s_ba);
-    uint32_t c = background;
-    if (a != 0) {
-      const uint32_t r = min(static_cast<uint32_t>(s_rg >> 32) / a, 255u);
-      const uint32_t g = min(static_cast<uint32_t>(s_rg) / a, 255u);
-      const uint32_t b = min(static_cast<uint32_t>(s_ba >> 32) / a, 255u);
-      c = r | (g << 8) | (b << 16) | 0xFF000000u;
-    }
-    out[p] = c;
+    out[p] = average_color(static_cast<uint32_t>(s_rg >> 32), static_cast<uint32_t>(s_rg),
+                           static_cast<uint32_t>(s_ba >> 32), static_cast<uint32_t>(s_ba), background);
   }
 }
 
@@ -476,14 +469,10 @@ __global__ void k_resolve_hq1r(const unsigned long long* __restrict__ primary, c
     const unsigned long long s_rg = rg[p];
     const unsigned long long s_ba = ba[p];
     const uint32_t a = static_cast<uint32_t>(s_ba) + static_cast<uint32_t>(w1 & kHq1rCountMask);
-    uint32_t c = background;
-    if (a != 0) {
-      const uint32_t sr = static_cast<uint32_t>(s_rg >> 32) + static_cast<uint32_t>((w1 >> kHq1rShiftR) & kHq1rChannelMask);
-      const uint32_t sg = static_cast<uint32_t>(s_rg) + static_cast<uint32_t>((w1 >> kHq1rShiftG) & kHq1rChannelMask);
-      const uint32_t sb = static_cast<uint32_t>(s_ba >> 32) + static_cast<uint32_t>((w1 >> kHq1rShiftB) & kHq1rChannelMask);
-      c = min(sr / a, 255u) | (min(sg / a, 255u) << 8) | (min(sb / a, 255u) << 16) | 0xFF000000u;
-    }
-    out[p] = c;
+    const uint32_t sr = static_cast<uint32_t>(s_rg >> 32) + static_cast<uint32_t>((w1 >> kHq1rShiftR) & kHq1rChannelMask);
+    const uint32_t sg = static_cast<uint32_t>(s_rg) + static_cast<uint32_t>((w1 >> kHq1rShiftG) & kHq1rChannelMask);
+    const uint32_t sb = static_cast<uint32_t>(s_ba >> 32) + static_cast<uint32_t>((w1 >> kHq1rShiftB) & kHq1rChannelMask);
+    out[p] = average_color(sr, sg, sb, a, background);
   }
 }
 
@@ -614,16 +603,17 @@ cudaError_t launch_hq_depth(int variant, const uint4* pts, uint32_t n, const Vie
 }
 
 template <bool AGG, bool V8>
-void launch_color_k(const uint4* pts, uint32_t n, const ViewParams& v, float depth_factor, const uint32_t* depth,
+void launch_color_k(const uint4* pts, uint32_t n, const ViewParams& v, float depth_factor, DepthSource depth,
                     unsigned long long* rg, unsigned long long* ba, cudaStream_t s, const Device& d) {
   constexpr auto k = k_hq_color<AGG, kUnroll, V8>;
   k<<<geometry_grid<k, kUnroll>(n, d), kThreads, 0, s>>>(pts, n, v, depth_factor, depth, rg, ba);
 }
 
 cudaError_t launch_hq_color(int variant, const uint4* pts, uint32_t n, const ViewParams& v, float depth_factor,
-                            const uint32_t* depth, unsigned long long* rg, unsigned long long* ba, cudaStream_t s,
-                            const Device& d) {
+                            const uint32_t* depth_base, uint32_t depth_step, unsigned long long* rg,
+                            unsigned long long* ba, cudaStream_t s, const Device& d) {
   if (n == 0) return cudaSuccess;
+  const DepthSource depth{depth_base, depth_step};
   // every variant but the basic one groups colours before adding
   const bool agg = variant != PCR_VARIANT_ATOMICMIN;
   if (!agg) launch_color_k<false, false>(pts, n, v, depth_factor, depth, rg, ba, s, d);
@@ -662,7 +652,7 @@ void prewarm_single_view(const Device& d) {
 }
 
 template <bool AGG, bool V8>
-void launch_hq1r_k(const uint4* pts, uint32_t n, const ViewParams& v, float depth_factor, const uint32_t* depth,
+void launch_hq1r_k(const uint4* pts, uint32_t n, const ViewParams& v, float depth_factor, DepthSource depth,
                    unsigned long long* primary, unsigned long long* rg, unsigned long long* ba, cudaStream_t s,
                    const Device& d) {
   constexpr auto k = k_hq1r_color<AGG, kUnroll, V8>;
@@ -670,9 +660,10 @@ void launch_hq1r_k(const uint4* pts, uint32_t n, const ViewParams& v, float dept
 }
 
 cudaError_t launch_hq1r_color(int variant, const uint4* pts, uint32_t n, const ViewParams& v, float depth_factor,
-                              const uint32_t* depth, unsigned long long* primary, unsigned long long* rg,
+                              const uint32_t* depth_base, unsigned long long* primary, unsigned long long* rg,
                               unsigned long long* ba, cudaStream_t s, const Device& d) {
   if (n == 0) return cudaSuccess;
+  const DepthSource depth{depth_base, sizeof(uint32_t)};
   const bool agg = variant != PCR_VARIANT_ATOMICMIN;
   if (!agg) launch_hq1r_k<false, false>(pts, n, v, depth_factor, depth, primary, rg, ba, s, d);
   else if (pairs_aligned(pts)) launch_hq1r_k<true, kCanPairLoad>(pts, n, v, depth_factor, depth, primary, rg, ba, s, d);

@@ -287,3 +287,29 @@ def test_batch_random_descriptions(ctx, oracle, seed):
     _poison(bufs)
     pcr.pcr_batch_launch(ctx, ws, config)
     _check(bufs, expected, f"seed {seed} config {config}")
+
+
+@pytest.mark.parametrize("shift", (0, 1, 2, 3))
+def test_batch_buffers_at_element_alignment(ctx, oracle, shift):
+    """Views' buffers that start `shift` elements past a 16-byte boundary, with
+    sizes on both sides of a multiple of four pixels and of a screen tile."""
+    cloud = scenes.random_cloud(9001, seed=3).numpy()
+    views = []
+    for k, (W, H) in enumerate(((64, 64), (61, 67), (63, 65), (4097, 1), (3, 1), (1, 1))):
+        m = scenes.camera((2.5, 0.3 * k, 1.0), (0, 0, 0), (0, 0, 1), W, H)
+        views.append((0, m, W, H, (BASIC | HQ, BASIC, HQ)[k % 3]))
+    expected = _expected(oracle, [cloud], views)
+    dev = torch.from_numpy(cloud.copy()).cuda()
+    bufs, vs = [], []
+    for (c, m, W, H, flags) in views:
+        b = {k: torch.empty(W * H + shift, dtype=t.dtype, device="cuda")[shift:] for k, t in _buffers(W, H).items()}
+        kw = {k: b[k] for k in (("keys", "image") if flags & BASIC else ()) +
+              (("hq_depth", "hq_rg", "hq_ba", "hq_image") if flags & HQ else ())}
+        bufs.append(b)
+        vs.append(pcr.batch_view(m, W, H, c, flags, **kw))
+    ws = torch.empty(pcr.pcr_batch_workspace_size(), dtype=torch.uint8, device="cuda")
+    pcr.pcr_batch_prepare(ctx, [pcr.batch_cloud(dev)], vs, 1.01, BG, ws)
+    for config in (0, 8):
+        _poison(bufs)
+        pcr.pcr_batch_launch(ctx, ws, config)
+        _check(bufs, expected, f"shift {shift} config {config}")

@@ -466,3 +466,29 @@ def test_captured_frames_replay_exactly(oracle):
         assert pcr.pcr_last_device_error(h) == 0  # the context is usable again after the capture
     with pcr.Context(0, stream=torch.cuda.current_stream()) as c2:
         pcr.pcr_capture_begin(c2.handle)  # left open: pcr_destroy drops it
+
+
+@pytest.mark.parametrize("scale", (1, 255, 4096, 2**24, 2**32 - 1))
+def test_hq_resolve_averages_are_exact_divisions(r, oracle, scale):
+    """The resolve's reciprocal and remainder against integer division: counts
+    and sums over the whole 32-bit range, and sums next to multiples of their
+    count (0 to 256 times it)."""
+    rng = np.random.default_rng(scale % 1000)
+    n = 250 * 200
+    a = rng.integers(1, scale + 1, n, dtype=np.uint64)
+    a[:50] = [1, 2, 3, scale, max(scale - 1, 1)] * 10
+    a[50:60] = 0
+    q = rng.integers(0, 257, (3, n)).astype(np.uint64)
+    s = np.minimum(np.where(rng.random((3, n)) < 0.8, q * a + rng.integers(-1, 2, (3, n)).astype(np.int64).astype(np.uint64),
+                            rng.integers(0, 2**32, (3, n), dtype=np.uint64)), np.uint64(2**32 - 1))
+    s = np.where(s > 2**63, np.uint64(0), s)
+    rg = (s[0] << np.uint64(32)) | s[1]
+    ba = (s[2] << np.uint64(32)) | a
+    r.upload(scenes.random_cloud(10, seed=1).numpy())
+    r.view(scenes.camera((0, 0, 4), (0, 0, 0), (0, 1, 0), 250, 200), 250, 200)
+    r.fb["hq_rg"].copy_(torch.from_numpy(rg.view(np.int64)))
+    r.fb["hq_ba"].copy_(torch.from_numpy(ba.view(np.int64)))
+    r.fb["hq1r_primary"].zero_()
+    expect = oracle.resolve_hq(rg, ba, BG)
+    assert np.array_equal(r.resolve(pcr.PCR_RESOLVE_HQ, BG), expect)
+    assert np.array_equal(r.resolve(pcr.PCR_RESOLVE_HQ1R, BG), expect)
