@@ -219,6 +219,7 @@ __device__ __forceinline__ void project_all(const ViewParams& vp, const uint4 (&
 // keys alone, 20.6 with deduplication).
 template <int U, int T>
 __global__ void __launch_bounds__(T) k_batch_phase1(const Tables* __restrict__ tables) {
+  after_previous();
   const Shared sh = load_tables(tables, 0);
   const uint64_t pol_stream = policy_evict_first();
   const uint64_t pol_fb = policy_evict_last();
@@ -257,6 +258,7 @@ __global__ void __launch_bounds__(T) k_batch_phase1(const Tables* __restrict__ t
 // Held to 64 registers (1024 threads per SM) at either block size.
 template <int U, int T>
 __global__ void __launch_bounds__(T, 1024 / T) k_batch_phase2(const Tables* __restrict__ tables) {
+  after_previous();
   const Shared sh = load_tables(tables, 1);
   const uint64_t pol_stream = policy_evict_first();
   const uint64_t pol_fb = policy_evict_last();
@@ -330,6 +332,7 @@ __device__ __forceinline__ void load_words(const unsigned long long* p, unsigned
 }
 
 __global__ void __launch_bounds__(kThreads) k_batch_clear(const Tables* __restrict__ tables) {
+  after_previous();
   const Shared sh = load_tables(tables, -1);
   for_each_pixel_group(sh, [&](const BatchView& bv, uint64_t q, int count) {
     if (bv.flags & PCR_BATCH_BASIC) fill_words(bv.keys + q, kEmptyKey, count);
@@ -344,6 +347,7 @@ __global__ void __launch_bounds__(kThreads) k_batch_clear(const Tables* __restri
 // Images, and the depth buffers of views whose depths are their keys' (see
 // k_batch_phase1).
 __global__ void __launch_bounds__(kThreads) k_batch_resolve(const Tables* __restrict__ tables) {
+  after_previous();
   const Shared sh = load_tables(tables, -1);
   const uint32_t background = sh.hdr.background;
   for_each_pixel_group(sh, [&](const BatchView& bv, uint64_t q, int count) {
@@ -405,25 +409,26 @@ int batch_resident(int threads, uint32_t smem) {
 }
 
 template <auto K, int T>
-void launch_persistent(const Tables* t, uint32_t smem, cudaStream_t s, const Device& d) {
-  K<<<d.num_sms * batch_resident<K>(T, smem), T, smem, s>>>(t);
+cudaError_t launch_persistent(const Tables* t, uint32_t smem, cudaStream_t s, const Device& d) {
+  return launch_kernel(K, d.num_sms * batch_resident<K>(T, smem), T, smem, s, t);
 }
 
 template <int T>
-void launch_phase(const Tables* t, uint32_t smem, int config, int phase, cudaStream_t s, const Device& d) {
+cudaError_t launch_phase(const Tables* t, uint32_t smem, int config, int phase, cudaStream_t s, const Device& d) {
   if (phase == 0) {
-    if (config & 2) launch_persistent<k_batch_phase1<2, T>, T>(t, smem, s, d);
-    else launch_persistent<k_batch_phase1<4, T>, T>(t, smem, s, d);
-  } else {
-    if (config & 1) launch_persistent<k_batch_phase2<2, T>, T>(t, smem, s, d);
-    else launch_persistent<k_batch_phase2<4, T>, T>(t, smem, s, d);
+    if (config & 2) return launch_persistent<k_batch_phase1<2, T>, T>(t, smem, s, d);
+    return launch_persistent<k_batch_phase1<4, T>, T>(t, smem, s, d);
+  }
+  {
+    if (config & 1) return launch_persistent<k_batch_phase2<2, T>, T>(t, smem, s, d);
+    return launch_persistent<k_batch_phase2<4, T>, T>(t, smem, s, d);
   }
 }
 
-void launch_batch_phase(const Tables& h, const Tables* t, int config, int phase, cudaStream_t s, const Device& d) {
+cudaError_t launch_batch_phase(const Tables& h, const Tables* t, int config, int phase, cudaStream_t s, const Device& d) {
   const uint32_t smem = shared_layout(h.hdr.num_clouds, h.hdr.num_views, h.hdr.num_groups[phase], true).bytes;
-  if (config & 4) launch_phase<512>(t, smem, config, phase, s, d);
-  else launch_phase<256>(t, smem, config, phase, s, d);
+  if (config & 4) return launch_phase<512>(t, smem, config, phase, s, d);
+  return launch_phase<256>(t, smem, config, phase, s, d);
 }
 
 // The single-view kernels of one view and phase (index): 0 the basic keys
@@ -630,25 +635,17 @@ cudaError_t batch_launch(const void* host_tables, const void* workspace, int con
   const Tables* t = static_cast<const Tables*>(workspace);
   const int screen_blocks = d.num_sms * 8;
   const uint32_t screen_smem = shared_layout(h.hdr.num_clouds, h.hdr.num_views, 0, false).bytes;
-  k_batch_clear<<<screen_blocks, kThreads, screen_smem, s>>>(t);
-  cudaError_t e = cudaGetLastError();
-  if (e == cudaSuccess && h.hdr.total_slots[0] > 0) {
-    launch_batch_phase(h, t, config, 0, s, d);
-    e = cudaGetLastError();
-  }
+  cudaError_t e = launch_kernel(k_batch_clear, screen_blocks, kThreads, screen_smem, s, t);
+  if (e == cudaSuccess && h.hdr.total_slots[0] > 0) e = launch_batch_phase(h, t, config, 0, s, d);
   for (uint32_t k = 0; k < h.num_single[0] && e == cudaSuccess; ++k) e = launch_single(h, h.single[0][k], 0, s, d);
   if (batch_config_single_colors(config)) {
     for (uint32_t vi = 0; vi < h.hdr.num_views && e == cudaSuccess; ++vi) e = launch_single(h, vi, 1, s, d);
   } else {
-    if (e == cudaSuccess && h.hdr.total_slots[1] > 0) {
-      launch_batch_phase(h, t, config, 1, s, d);
-      e = cudaGetLastError();
-    }
+    if (e == cudaSuccess && h.hdr.total_slots[1] > 0) e = launch_batch_phase(h, t, config, 1, s, d);
     for (uint32_t k = 0; k < h.num_single[1] && e == cudaSuccess; ++k) e = launch_single(h, h.single[1][k], 1, s, d);
   }
   if (e != cudaSuccess) return e;
-  k_batch_resolve<<<screen_blocks, kThreads, screen_smem, s>>>(t);
-  return cudaGetLastError();
+  return launch_kernel(k_batch_resolve, screen_blocks, kThreads, screen_smem, s, t);
 }
 
 }  // namespace pcr

@@ -328,4 +328,18 @@ __device__ __forceinline__ unsigned long long atom_exch_u64(unsigned long long* 
 
 __device__ __forceinline__ uint32_t lane_id() { return threadIdx.x & 31u; }
 
+// Start of every kernel (see launch_kernel): returns once the previous kernel
+// of the stream, and so everything before it, has finished and its writes are
+// visible; no kernel touches global memory before.  The branch, never taken,
+// keeps the compiler from moving loads it takes for constant (of const
+// __restrict__ parameters) above the wait: past it they would be speculative.
+__device__ __forceinline__ void after_previous() {
+  uint32_t never;
+  asm volatile("griddepcontrol.wait;\n\tmov.u32 %0, 0;" : "=r"(never)::"memory");
+  if (never != 0u) {
+    asm volatile("exit;");
+    __builtin_unreachable();
+  }
+}
+
 }  // namespace pcr

@@ -2,6 +2,7 @@
 #pragma once
 
 #include <cstdint>
+#include <utility>
 #include <cuda_runtime.h>
 
 #include "../../include/pcr.h"
@@ -13,6 +14,41 @@ namespace pcr {
 struct Device {
   int id = 0;
   int num_sms = 0;
+};
+
+// Launch a kernel whose blocks may start as the blocks of the stream's previous
+// kernel end.  Every kernel launched so begins with after_previous() in every
+// thread, so its work starts where a plain launch's would; what overlaps is
+// the launch itself: a 1M-point frame of three launches 19.0 -> 12.3 us, 20k
+// points 11.9 -> 7.6, the seven launches of a 100k-point reorder 67 -> 48.
+// No kernel lets the next one start before its own end
+// (griddepcontrol.launch_dependents): waiting blocks then only stand in the
+// way (12.8, 7.6 and 50 us; a 2M-point reorder 278 against 231).
+template <class... P, class... A>
+cudaError_t launch_kernel(void (*kernel)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t s, A&&... args) {
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t c{};
+  c.gridDim = grid;
+  c.blockDim = dim3(threads);
+  c.dynamicSmemBytes = smem;
+  c.stream = s;
+  c.attrs = &attr;
+  c.numAttrs = 1;
+  const cudaError_t e = cudaLaunchKernelEx(&c, kernel, std::forward<A>(args)...);
+  if (e != cudaSuccess) cudaGetLastError();  // leave no error behind for the next call to find
+  return e;
+}
+
+// A sequence of launches on one stream that ends at its first error.
+struct LaunchChain {
+  cudaStream_t stream;
+  cudaError_t error = cudaSuccess;
+  template <class K, class... A>
+  void operator()(K kernel, dim3 grid, unsigned threads, size_t smem, A&&... args) {
+    if (error == cudaSuccess) error = launch_kernel(kernel, grid, threads, smem, stream, std::forward<A>(args)...);
+  }
 };
 
 cudaError_t launch_fill_u64(unsigned long long* p, uint64_t count, unsigned long long value, cudaStream_t s,

@@ -115,6 +115,7 @@ __device__ __forceinline__ uint32_t bucket_of(uint32_t key, uint32_t buckets) { 
 __device__ __forceinline__ uint32_t place_of(uint32_t key, uint32_t buckets) { return key * buckets; }
 
 __global__ void __launch_bounds__(256) k_zero_words(uint32_t* __restrict__ p, uint64_t count) {
+  after_previous();
   for (uint64_t i = blockIdx.x * 256ull + threadIdx.x; i < count; i += gridDim.x * 256ull) p[i] = 0u;
 }
 
@@ -122,6 +123,7 @@ __global__ void __launch_bounds__(256) k_zero_words(uint32_t* __restrict__ p, ui
 __global__ void __launch_bounds__(kPartThreads) k_random_count_first(uint32_t count, uint64_t seed, uint32_t buckets,
                                                                      int second, uint32_t radix,
                                                                      uint32_t* __restrict__ counts) {
+  after_previous();
   extern __shared__ __align__(16) uint32_t s_count[];
   for (uint32_t d = threadIdx.x; d < radix; d += kPartThreads) s_count[d] = 0u;
   __syncthreads();
@@ -140,6 +142,7 @@ constexpr uint32_t kCountChunk = 16384;
 __global__ void __launch_bounds__(kPartThreads) k_random_count_second(const uint32_t* __restrict__ iin, uint32_t count,
                                                                       uint64_t seed, uint32_t buckets, int second,
                                                                       uint32_t* __restrict__ counts) {
+  after_previous();
   extern __shared__ __align__(16) uint32_t s_count[];
   const uint32_t radix = 1u << second;
   const uint64_t first = blockIdx.x * static_cast<uint64_t>(kCountChunk);
@@ -179,6 +182,7 @@ __global__ void __launch_bounds__(kPartThreads, 2)
     k_random_partition(const uint4* __restrict__ rin, const uint32_t* __restrict__ iin, uint4* __restrict__ rout,
                        uint32_t* __restrict__ iout, uint32_t n, uint64_t seed, uint32_t buckets, int second,
                        uint32_t radix, uint32_t* __restrict__ cursors) {
+  after_previous();
   extern __shared__ __align__(16) unsigned char s_bytes[];
   uint4* s_rec = reinterpret_cast<uint4*>(s_bytes);                                      // [kPartTile] with REC
   uint32_t* s_idx = reinterpret_cast<uint32_t*>(s_bytes + (REC ? sizeof(uint4) * kPartTile : 0));  // [kPartTile]
@@ -290,6 +294,7 @@ template <bool REC>
 __global__ void __launch_bounds__(kFinishThreads, 4)
     k_random_finish(const uint4* rin, const uint32_t* __restrict__ iin, uint32_t n, uint64_t seed, uint32_t buckets,
                     const uint32_t* __restrict__ ends, RandomOut out, uint4* spare) {
+  after_previous();
   extern __shared__ __align__(16) unsigned char s_bytes[];
   uint4* s_rec = reinterpret_cast<uint4*>(s_bytes);
   uint32_t* s_word = reinterpret_cast<uint32_t*>(s_bytes + (REC ? sizeof(uint4) * kFinishCap : 0));
@@ -439,10 +444,10 @@ template <bool REC>
 cudaError_t random_order(uint4* pts, uint4* copy, uint32_t n, uint64_t seed, uint32_t* const idx[2],
                          uint32_t* counters, uint32_t* partials, RandomOut out, cudaStream_t s, const Device& d) {
   const RandomSplit p = random_split(n);
-  cudaError_t e = cudaSuccess;
+  LaunchChain run{s};
   auto allow = [&](auto kernel, size_t bytes) {
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
+    if (run.error == cudaSuccess)
+      run.error = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
   };
   const uint4* rin = pts;
   const uint32_t* iin = nullptr;
@@ -452,15 +457,13 @@ cudaError_t random_order(uint4* pts, uint4* copy, uint32_t n, uint64_t seed, uin
     const uint32_t tiles = static_cast<uint32_t>((static_cast<uint64_t>(n) + kPartTile - 1) / kPartTile);
     const uint32_t radix = first_digits(p);
     uint32_t* first = counters;
-    k_zero_words<<<static_cast<unsigned>(words / 256 + 1 < 256 ? words / 256 + 1 : 256), 256, 0, s>>>(counters, words);
+    run(k_zero_words, static_cast<unsigned>(words / 256 + 1 < 256 ? words / 256 + 1 : 256), 256, 0, counters, words);
     const uint32_t blocks = tiles < 4u * d.num_sms ? tiles : 4u * d.num_sms;
-    k_random_count_first<<<blocks, kPartThreads, sizeof(uint32_t) * radix, s>>>(n, seed, p.buckets, p.second, radix,
+    run(k_random_count_first, blocks, kPartThreads, sizeof(uint32_t) * radix, n, seed, p.buckets, p.second, radix,
                                                                                first);
-    k_scan_partials<<<1, 1024, 0, s>>>(first, radix);
+    run(k_scan_partials, 1, 1024, 0, first, radix);
     allow(k_random_partition<REC, true>, partition_smem<REC>(radix));
-    if (e != cudaSuccess) return e;
-    k_random_partition<REC, true><<<tiles, kPartThreads, partition_smem<REC>(radix), s>>>(
-        pts, nullptr, copy, idx[0], n, seed, p.buckets, p.second, radix, first);
+    run(k_random_partition<REC, true>, tiles, kPartThreads, partition_smem<REC>(radix), pts, nullptr, copy, idx[0], n, seed, p.buckets, p.second, radix, first);
     rin = copy;
     iin = idx[0];
     ends = first;
@@ -468,13 +471,11 @@ cudaError_t random_order(uint4* pts, uint4* copy, uint32_t n, uint64_t seed, uin
       uint32_t* both = counters + second_counters(p);
       const uint32_t low = second_digits(p);
       const uint32_t chunks = static_cast<uint32_t>((static_cast<uint64_t>(n) + kCountChunk - 1) / kCountChunk);
-      k_random_count_second<<<chunks, kPartThreads, sizeof(uint32_t) * low, s>>>(idx[0], n, seed, p.buckets, p.second,
+      run(k_random_count_second, chunks, kPartThreads, sizeof(uint32_t) * low, idx[0], n, seed, p.buckets, p.second,
                                                                                 both);
-      e = exclusive_scan(both, p.buckets, partials, s);
+      if (run.error == cudaSuccess) run.error = exclusive_scan(both, p.buckets, partials, s);
       allow(k_random_partition<REC, false>, partition_smem<REC>(low));
-      if (e != cudaSuccess) return e;
-      k_random_partition<REC, false><<<tiles, kPartThreads, partition_smem<REC>(low), s>>>(
-          copy, idx[0], pts, idx[1], n, seed, p.buckets, p.second, low, both);
+      run(k_random_partition<REC, false>, tiles, kPartThreads, partition_smem<REC>(low), copy, idx[0], pts, idx[1], n, seed, p.buckets, p.second, low, both);
       rin = pts;
       iin = idx[1];
       ends = both;
@@ -482,10 +483,9 @@ cudaError_t random_order(uint4* pts, uint4* copy, uint32_t n, uint64_t seed, uin
   }
   out.dst = pts;
   allow(k_random_finish<REC>, finish_smem<REC>());
-  if (e != cudaSuccess) return e;
-  k_random_finish<REC><<<p.buckets, kFinishThreads, finish_smem<REC>(), s>>>(rin, iin, n, seed, p.buckets, ends, out,
+  run(k_random_finish<REC>, p.buckets, kFinishThreads, finish_smem<REC>(), rin, iin, n, seed, p.buckets, ends, out,
                                                                               copy);
-  return cudaGetLastError();
+  return run.error;
 }
 
 }  // namespace

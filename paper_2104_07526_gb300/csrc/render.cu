@@ -86,6 +86,7 @@ constexpr int kHqMinBlocks = kMinBlocks < 6 ? 6 : kMinBlocks;
 template <int V, int U, int P>
 __global__ void __launch_bounds__(kThreads, kRenderMinBlocks) k_render_basic(const uint4* __restrict__ pts, uint32_t n, ViewParams v,
                                                            unsigned long long* __restrict__ fb) {
+  after_previous();
   constexpr int L = kInterleaved;
   const uint64_t pol_stream = policy_evict_first();
   const uint64_t pol_fb = policy_evict_last();
@@ -177,6 +178,7 @@ template <int U>
 __global__ void __launch_bounds__(kThreads, kMinBlocks) k_render_busy(const uint4* __restrict__ pts, uint32_t n, ViewParams v,
                                                           unsigned long long* __restrict__ fb,
                                                           uint32_t* __restrict__ locks, uint64_t limit_ns) {
+  after_previous();
   const uint64_t pol_stream = policy_evict_first();
   for_each_chunk<U, kInterleaved, false>(pts, n, pol_stream, [&](const uint4(&r)[U], uint32_t base, auto full) {
     uint32_t pix[U];
@@ -204,6 +206,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) k_render_busy(const uint
 template <int V, int U>
 __global__ void __launch_bounds__(kThreads, kHqMinBlocks) k_hq_depth(const uint4* __restrict__ pts, uint32_t n, ViewParams v,
                                                        uint32_t* __restrict__ depth) {
+  after_previous();
   constexpr int L = kInterleaved;
   const uint64_t pol_stream = policy_evict_first();
   const uint64_t pol_fb = policy_evict_last();
@@ -241,6 +244,7 @@ __global__ void __launch_bounds__(kThreads, kHqMinBlocks) k_hq_color(const uint4
                                                        float factor, DepthSource depth,
                                                        unsigned long long* __restrict__ rg,
                                                        unsigned long long* __restrict__ ba) {
+  after_previous();
   const uint64_t pol_stream = policy_evict_first();
   const uint64_t pol_fb = policy_evict_last();
   constexpr int L = AGG ? kConsecutive : kInterleaved;
@@ -338,6 +342,7 @@ __global__ void __launch_bounds__(kThreads, PCR_HQ1R_MIN_BLOCKS)
     k_hq1r_color(const uint4* __restrict__ pts, uint32_t n, ViewParams v, float factor,
                  DepthSource depth, unsigned long long* __restrict__ primary,
                  unsigned long long* __restrict__ rg, unsigned long long* __restrict__ ba) {
+  after_previous();
   const uint64_t pol_stream = policy_evict_first();
   const uint64_t pol_fb = policy_evict_last();
   constexpr int L = AGG ? kConsecutive : kInterleaved;
@@ -395,6 +400,7 @@ __global__ void __launch_bounds__(kThreads, PCR_HQ1R_MIN_BLOCKS)
 // ---------------------------------------------------------------------------
 
 __global__ void k_fill_u64(unsigned long long* __restrict__ p, uint64_t count, unsigned long long value) {
+  after_previous();
   for (uint64_t i = blockIdx.x * static_cast<uint64_t>(blockDim.x) + threadIdx.x; i < count;
        i += static_cast<uint64_t>(gridDim.x) * blockDim.x)
     p[i] = value;
@@ -402,6 +408,7 @@ __global__ void k_fill_u64(unsigned long long* __restrict__ p, uint64_t count, u
 
 __global__ void k_clear_hq(uint32_t* __restrict__ depth, unsigned long long* __restrict__ rg,
                            unsigned long long* __restrict__ ba, uint64_t npx) {
+  after_previous();
   for (uint64_t i = blockIdx.x * static_cast<uint64_t>(blockDim.x) + threadIdx.x; i < npx;
        i += static_cast<uint64_t>(gridDim.x) * blockDim.x) {
     depth[i] = kInfBits;
@@ -415,6 +422,7 @@ __global__ void k_clear_hq(uint32_t* __restrict__ depth, unsigned long long* __r
 __global__ void k_resolve_basic(const unsigned long long* __restrict__ keys, uint64_t npx,
                                 const uint32_t* __restrict__ words, uint32_t n, uint32_t background,
                                 uint32_t* __restrict__ out) {
+  after_previous();
   for (uint64_t p = blockIdx.x * static_cast<uint64_t>(blockDim.x) + threadIdx.x; p < npx;
        p += static_cast<uint64_t>(gridDim.x) * blockDim.x) {
     const unsigned long long k = keys[p];
@@ -434,6 +442,7 @@ __global__ void k_resolve_basic(const unsigned long long* __restrict__ keys, uin
 // key's low 24 bits; alpha 255.
 __global__ void k_resolve_rgb(const unsigned long long* __restrict__ keys, uint64_t npx, uint32_t background,
                               uint32_t* __restrict__ out) {
+  after_previous();
   for (uint64_t p = blockIdx.x * static_cast<uint64_t>(blockDim.x) + threadIdx.x; p < npx;
        p += static_cast<uint64_t>(gridDim.x) * blockDim.x) {
     const unsigned long long k = keys[p];
@@ -442,6 +451,7 @@ __global__ void k_resolve_rgb(const unsigned long long* __restrict__ keys, uint6
 }
 
 __global__ void k_fill_u32(uint32_t* __restrict__ p, uint64_t count, uint32_t value) {
+  after_previous();
   for (uint64_t i = blockIdx.x * static_cast<uint64_t>(blockDim.x) + threadIdx.x; i < count;
        i += static_cast<uint64_t>(gridDim.x) * blockDim.x)
     p[i] = value;
@@ -450,6 +460,7 @@ __global__ void k_fill_u32(uint32_t* __restrict__ p, uint64_t count, uint32_t va
 // Sec. 3.5, Listing "hqs_resolve": truncating average, alpha 255.
 __global__ void k_resolve_hq(const unsigned long long* __restrict__ rg, const unsigned long long* __restrict__ ba,
                              uint64_t npx, uint32_t background, uint32_t* __restrict__ out) {
+  after_previous();
   for (uint64_t p = blockIdx.x * static_cast<uint64_t>(blockDim.x) + threadIdx.x; p < npx;
        p += static_cast<uint64_t>(gridDim.x) * blockDim.x) {
     const unsigned long long s_rg = rg[p];
@@ -463,6 +474,7 @@ __global__ void k_resolve_hq(const unsigned long long* __restrict__ rg, const un
 __global__ void k_resolve_hq1r(const unsigned long long* __restrict__ primary, const unsigned long long* __restrict__ rg,
                                const unsigned long long* __restrict__ ba, uint64_t npx, uint32_t background,
                                uint32_t* __restrict__ out) {
+  after_previous();
   for (uint64_t p = blockIdx.x * static_cast<uint64_t>(blockDim.x) + threadIdx.x; p < npx;
        p += static_cast<uint64_t>(gridDim.x) * blockDim.x) {
     const unsigned long long w1 = primary[p];
@@ -514,8 +526,7 @@ template <int V, int P>
 cudaError_t launch_basic_v(const uint4* pts, uint32_t n, const ViewParams& v, unsigned long long* keys, cudaStream_t s,
                            const Device& d) {
   constexpr auto k = k_render_basic<V, kUnroll, P>;
-  k<<<geometry_grid<k, kUnroll>(n, d), kThreads, 0, s>>>(pts, n, v, keys);
-  return cudaGetLastError();
+  return launch_kernel(k, geometry_grid<k, kUnroll>(n, d), kThreads, 0, s, pts, n, v, keys);
 }
 
 template <int P>
@@ -537,8 +548,7 @@ template <int V>
 cudaError_t launch_depth_v(const uint4* pts, uint32_t n, const ViewParams& v, uint32_t* depth, cudaStream_t s,
                            const Device& d) {
   constexpr auto k = k_hq_depth<V, kUnroll>;
-  k<<<geometry_grid<k, kUnroll>(n, d), kThreads, 0, s>>>(pts, n, v, depth);
-  return cudaGetLastError();
+  return launch_kernel(k, geometry_grid<k, kUnroll>(n, d), kThreads, 0, s, pts, n, v, depth);
 }
 
 }  // namespace
@@ -546,15 +556,13 @@ cudaError_t launch_depth_v(const uint4* pts, uint32_t n, const ViewParams& v, ui
 cudaError_t launch_fill_u64(unsigned long long* p, uint64_t count, unsigned long long value, cudaStream_t s,
                             const Device& d) {
   if (count == 0) return cudaSuccess;
-  k_fill_u64<<<screen_grid(count, d), kThreads, 0, s>>>(p, count, value);
-  return cudaGetLastError();
+  return launch_kernel(k_fill_u64, screen_grid(count, d), kThreads, 0, s, p, count, value);
 }
 
 cudaError_t launch_clear_hq(uint32_t* depth, unsigned long long* rg, unsigned long long* ba, uint64_t npx,
                             cudaStream_t s, const Device& d) {
   if (npx == 0) return cudaSuccess;
-  k_clear_hq<<<screen_grid(npx, d), kThreads, 0, s>>>(depth, rg, ba, npx);
-  return cudaGetLastError();
+  return launch_kernel(k_clear_hq, screen_grid(npx, d), kThreads, 0, s, depth, rg, ba, npx);
 }
 
 cudaError_t launch_render_basic(int variant, const uint4* pts, uint32_t n, const ViewParams& v,
@@ -573,21 +581,18 @@ cudaError_t launch_render_busy(const uint4* pts, uint32_t n, const ViewParams& v
                                uint32_t* locks, uint64_t limit_ns, cudaStream_t s, const Device& d) {
   if (n == 0) return cudaSuccess;
   constexpr auto k = k_render_busy<kUnroll>;
-  k<<<geometry_grid<k, kUnroll>(n, d), kThreads, 0, s>>>(pts, n, v, keys, locks, limit_ns);
-  return cudaGetLastError();
+  return launch_kernel(k, geometry_grid<k, kUnroll>(n, d), kThreads, 0, s, pts, n, v, keys, locks, limit_ns);
 }
 
 cudaError_t launch_fill_u32(uint32_t* p, uint64_t count, uint32_t value, cudaStream_t s, const Device& d) {
   if (count == 0) return cudaSuccess;
-  k_fill_u32<<<screen_grid(count, d), kThreads, 0, s>>>(p, count, value);
-  return cudaGetLastError();
+  return launch_kernel(k_fill_u32, screen_grid(count, d), kThreads, 0, s, p, count, value);
 }
 
 cudaError_t launch_resolve_rgb(const unsigned long long* keys, uint64_t npx, uint32_t background, uint32_t* out,
                                cudaStream_t s, const Device& d) {
   if (npx == 0) return cudaSuccess;
-  k_resolve_rgb<<<screen_grid(npx, d), kThreads, 0, s>>>(keys, npx, background, out);
-  return cudaGetLastError();
+  return launch_kernel(k_resolve_rgb, screen_grid(npx, d), kThreads, 0, s, keys, npx, background, out);
 }
 
 cudaError_t launch_hq_depth(int variant, const uint4* pts, uint32_t n, const ViewParams& v, uint32_t* depth,
@@ -603,10 +608,11 @@ cudaError_t launch_hq_depth(int variant, const uint4* pts, uint32_t n, const Vie
 }
 
 template <bool AGG, bool V8>
-void launch_color_k(const uint4* pts, uint32_t n, const ViewParams& v, float depth_factor, DepthSource depth,
+cudaError_t launch_color_k(const uint4* pts, uint32_t n, const ViewParams& v, float depth_factor, DepthSource depth,
                     unsigned long long* rg, unsigned long long* ba, cudaStream_t s, const Device& d) {
   constexpr auto k = k_hq_color<AGG, kUnroll, V8>;
-  k<<<geometry_grid<k, kUnroll>(n, d), kThreads, 0, s>>>(pts, n, v, depth_factor, depth, rg, ba);
+  return launch_kernel(k, geometry_grid<k, kUnroll>(n, d), kThreads, 0, s, pts, n, v, depth_factor, depth, rg,
+                       ba);
 }
 
 cudaError_t launch_hq_color(int variant, const uint4* pts, uint32_t n, const ViewParams& v, float depth_factor,
@@ -616,10 +622,9 @@ cudaError_t launch_hq_color(int variant, const uint4* pts, uint32_t n, const Vie
   const DepthSource depth{depth_base, depth_step};
   // every variant but the basic one groups colours before adding
   const bool agg = variant != PCR_VARIANT_ATOMICMIN;
-  if (!agg) launch_color_k<false, false>(pts, n, v, depth_factor, depth, rg, ba, s, d);
-  else if (pairs_aligned(pts)) launch_color_k<true, kCanPairLoad>(pts, n, v, depth_factor, depth, rg, ba, s, d);
-  else launch_color_k<true, false>(pts, n, v, depth_factor, depth, rg, ba, s, d);
-  return cudaGetLastError();
+  if (!agg) return launch_color_k<false, false>(pts, n, v, depth_factor, depth, rg, ba, s, d);
+  if (pairs_aligned(pts)) return launch_color_k<true, kCanPairLoad>(pts, n, v, depth_factor, depth, rg, ba, s, d);
+  return launch_color_k<true, false>(pts, n, v, depth_factor, depth, rg, ba, s, d);
 }
 
 template <int P>
@@ -652,11 +657,12 @@ void prewarm_single_view(const Device& d) {
 }
 
 template <bool AGG, bool V8>
-void launch_hq1r_k(const uint4* pts, uint32_t n, const ViewParams& v, float depth_factor, DepthSource depth,
+cudaError_t launch_hq1r_k(const uint4* pts, uint32_t n, const ViewParams& v, float depth_factor, DepthSource depth,
                    unsigned long long* primary, unsigned long long* rg, unsigned long long* ba, cudaStream_t s,
                    const Device& d) {
   constexpr auto k = k_hq1r_color<AGG, kUnroll, V8>;
-  k<<<geometry_grid<k, kUnroll>(n, d), kThreads, 0, s>>>(pts, n, v, depth_factor, depth, primary, rg, ba);
+  return launch_kernel(k, geometry_grid<k, kUnroll>(n, d), kThreads, 0, s, pts, n, v, depth_factor, depth,
+                       primary, rg, ba);
 }
 
 cudaError_t launch_hq1r_color(int variant, const uint4* pts, uint32_t n, const ViewParams& v, float depth_factor,
@@ -665,33 +671,29 @@ cudaError_t launch_hq1r_color(int variant, const uint4* pts, uint32_t n, const V
   if (n == 0) return cudaSuccess;
   const DepthSource depth{depth_base, sizeof(uint32_t)};
   const bool agg = variant != PCR_VARIANT_ATOMICMIN;
-  if (!agg) launch_hq1r_k<false, false>(pts, n, v, depth_factor, depth, primary, rg, ba, s, d);
-  else if (pairs_aligned(pts)) launch_hq1r_k<true, kCanPairLoad>(pts, n, v, depth_factor, depth, primary, rg, ba, s, d);
-  else launch_hq1r_k<true, false>(pts, n, v, depth_factor, depth, primary, rg, ba, s, d);
-  return cudaGetLastError();
+  if (!agg) return launch_hq1r_k<false, false>(pts, n, v, depth_factor, depth, primary, rg, ba, s, d);
+  if (pairs_aligned(pts)) return launch_hq1r_k<true, kCanPairLoad>(pts, n, v, depth_factor, depth, primary, rg, ba, s, d);
+  return launch_hq1r_k<true, false>(pts, n, v, depth_factor, depth, primary, rg, ba, s, d);
 }
 
 cudaError_t launch_resolve_hq1r(const unsigned long long* primary, const unsigned long long* rg,
                                 const unsigned long long* ba, uint64_t npx, uint32_t background, uint32_t* out,
                                 cudaStream_t s, const Device& d) {
   if (npx == 0) return cudaSuccess;
-  k_resolve_hq1r<<<screen_grid(npx, d), kThreads, 0, s>>>(primary, rg, ba, npx, background, out);
-  return cudaGetLastError();
+  return launch_kernel(k_resolve_hq1r, screen_grid(npx, d), kThreads, 0, s, primary, rg, ba, npx, background, out);
 }
 
 cudaError_t launch_resolve_basic(const unsigned long long* keys, uint64_t npx, const uint4* pts, uint32_t n,
                                  uint32_t background, uint32_t* out, cudaStream_t s, const Device& d) {
   if (npx == 0) return cudaSuccess;
-  k_resolve_basic<<<screen_grid(npx, d), kThreads, 0, s>>>(keys, npx, reinterpret_cast<const uint32_t*>(pts), n,
+  return launch_kernel(k_resolve_basic, screen_grid(npx, d), kThreads, 0, s, keys, npx, reinterpret_cast<const uint32_t*>(pts), n,
                                                            background, out);
-  return cudaGetLastError();
 }
 
 cudaError_t launch_resolve_hq(const unsigned long long* rg, const unsigned long long* ba, uint64_t npx,
                               uint32_t background, uint32_t* out, cudaStream_t s, const Device& d) {
   if (npx == 0) return cudaSuccess;
-  k_resolve_hq<<<screen_grid(npx, d), kThreads, 0, s>>>(rg, ba, npx, background, out);
-  return cudaGetLastError();
+  return launch_kernel(k_resolve_hq, screen_grid(npx, d), kThreads, 0, s, rg, ba, npx, background, out);
 }
 
 cudaError_t read_and_clear_debug_counts(uint64_t out[4], cudaStream_t s, bool* available) {

@@ -143,6 +143,7 @@ __device__ __forceinline__ float order_float(uint32_t o) {
 }
 
 __global__ void k_bounds_init(uint32_t* misc) {
+  after_previous();
   if (threadIdx.x < 3) {
     misc[threadIdx.x] = 0xFF800000u;     // order of +inf: identity for min
     misc[3 + threadIdx.x] = 0x007FFFFFu; // order of -inf: identity for max
@@ -164,6 +165,7 @@ static_assert(kSortRounds % kMortonUnroll == 0, "whole rounds of records per til
 template <bool SMALL>
 __global__ void __launch_bounds__(256) k_bounds(const uint4* __restrict__ pts, uint32_t n, uint32_t* misc,
                                                 uint4* __restrict__ copy) {
+  after_previous();
   uint32_t lo[3] = {0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu};
   uint32_t hi[3] = {0u, 0u, 0u};
   // kStreamUnroll records per thread per step, all loads issued first
@@ -369,6 +371,7 @@ __global__ void __launch_bounds__(kSortThreads) k_morton(const uint4* __restrict
                                                          uint32_t* __restrict__ keys, uint32_t* __restrict__ counts,
                                                          uint32_t tiles, uint32_t parts,
                                                          ClearRows zero) {
+  after_previous();
   __shared__ TileKeys<ROUNDS> sh;
   constexpr uint32_t kT = kTileOf<ROUNDS>;
   zero_tile_hist(sh);
@@ -428,6 +431,7 @@ __global__ void __launch_bounds__(kSortThreads) k_morton63(const uint4* __restri
                                                            uint32_t* __restrict__ keys_lo, uint32_t* __restrict__ hi,
                                                            uint32_t* __restrict__ counts, uint32_t tiles, uint32_t parts,
                                                            ClearRows zero) {
+  after_previous();
   __shared__ TileKeys<ROUNDS> sh;
   constexpr uint32_t kT = kTileOf<ROUNDS>;
   zero_tile_hist(sh);
@@ -484,6 +488,7 @@ template <int ROUNDS, bool SMALL>
 __global__ void __launch_bounds__(kSortThreads) k_sort_hist(const uint32_t* __restrict__ keys, uint32_t n, int shift,
                                                             uint32_t* __restrict__ counts, uint32_t tiles,
                                                             ClearRows zero) {
+  after_previous();
   if constexpr (SMALL) clear_rows(zero);
   __shared__ uint32_t hist[kSortWarps][kRadix];
 #pragma unroll
@@ -587,6 +592,7 @@ __global__ void __launch_bounds__(kSortThreads, 4) k_sort_scatter(const uint32_t
                                                                   uint32_t tiles, const uint32_t* __restrict__ cin,
                                                                   uint32_t* __restrict__ cout, FinalGather fin,
                                                                   SmallPass small) {
+  after_previous();
   constexpr uint32_t kT = kTileOf<ROUNDS>;  // keys in a tile
   constexpr uint32_t kKeysPerWarp = kT / kSortWarps;
   extern __shared__ __align__(16) uint32_t smem[];
@@ -806,6 +812,7 @@ __device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t v, uint32_t& t
 
 __global__ void __launch_bounds__(kScanThreads) k_scan_reduce(const uint32_t* __restrict__ a, uint64_t len,
                                                               uint32_t* __restrict__ partials) {
+  after_previous();
   const uint64_t base = static_cast<uint64_t>(blockIdx.x) * kScanSeg + threadIdx.x;
   uint32_t s = 0;
 #pragma unroll
@@ -826,6 +833,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_reduce(const uint32_t* __
 
 // One block of 1024 threads; thread t scans a contiguous run of partials.
 __global__ void __launch_bounds__(1024) k_scan_partials(uint32_t* __restrict__ partials, uint32_t count) {
+  after_previous();
   const uint32_t per = (count + 1023) / 1024;
   const uint64_t first = static_cast<uint64_t>(threadIdx.x) * per;
   uint32_t local = 0;
@@ -848,6 +856,7 @@ __global__ void __launch_bounds__(1024) k_scan_partials(uint32_t* __restrict__ p
 // needed.
 __global__ void __launch_bounds__(kScanThreads) k_scan_down(uint32_t* __restrict__ a, uint64_t len,
                                                             const uint32_t* __restrict__ partials) {
+  after_previous();
   static_assert(kScanItems == 16, "four 16-byte vectors per thread");
   const uint64_t first = static_cast<uint64_t>(blockIdx.x) * kScanSeg + static_cast<uint64_t>(threadIdx.x) * kScanItems;
   uint32_t mine[kScanItems];
@@ -891,10 +900,11 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_down(uint32_t* __restrict
 
 cudaError_t exclusive_scan(uint32_t* a, uint64_t len, uint32_t* partials, cudaStream_t s) {
   const uint64_t blocks = ceil_div(len, kScanSeg);
-  k_scan_reduce<<<static_cast<unsigned>(blocks), kScanThreads, 0, s>>>(a, len, partials);
-  k_scan_partials<<<1, 1024, 0, s>>>(partials, static_cast<uint32_t>(blocks));
-  k_scan_down<<<static_cast<unsigned>(blocks), kScanThreads, 0, s>>>(a, len, partials);
-  return cudaGetLastError();
+  LaunchChain run{s};
+  run(k_scan_reduce, static_cast<unsigned>(blocks), kScanThreads, 0, a, len, partials);
+  run(k_scan_partials, 1, 1024, 0, partials, static_cast<uint32_t>(blocks));
+  run(k_scan_down, static_cast<unsigned>(blocks), kScanThreads, 0, a, len, partials);
+  return run.error;
 }
 
 // Stable sort of count (key, value) pairs on the low key_bits bits.  The
@@ -918,22 +928,20 @@ cudaError_t radix_sort(uint32_t* keys[2], uint32_t* vals[2], uint32_t count, int
   const uint32_t tiles = static_cast<uint32_t>(ceil_div(count, kTileOf<ROUNDS>));
   cudaError_t e = cudaFuncSetAttribute(k_sort_scatter<ROUNDS, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kSmem));
   if (e != cudaSuccess) return e;
+  LaunchChain run{s};
   for (int shift = 0; shift < key_bits; shift += kDigitBits) {
     const bool last = shift + kDigitBits >= key_bits;
-    if (!(first_counted && shift == 0)) k_sort_hist<ROUNDS, false><<<tiles, kSortThreads, 0, s>>>(keys[out], count, shift, counts, tiles, ClearRows{});
-    e = exclusive_scan(counts, static_cast<uint64_t>(kRadix) * tiles, partials, s);
-    if (e != cudaSuccess) return e;
+    if (!(first_counted && shift == 0)) run(k_sort_hist<ROUNDS, false>, tiles, kSortThreads, 0, keys[out], count, shift, counts, tiles, ClearRows{});
+    if (run.error == cudaSuccess) run.error = exclusive_scan(counts, static_cast<uint64_t>(kRadix) * tiles, partials, s);
     const uint32_t* vin = (index_values && shift == 0) ? nullptr : vals[out];
     uint32_t* kout = last ? nullptr : keys[out ^ 1];
     const FinalGather f = (last && fin) ? *fin : FinalGather{};
-    k_sort_scatter<ROUNDS, false><<<tiles, kSortThreads, kSmem, s>>>(
+    run(k_sort_scatter<ROUNDS, false>, tiles, kSortThreads, kSmem,
         keys[out], vin, kout, vals[out ^ 1], count, shift, counts, tiles, carry ? carry[out] : nullptr,
         carry ? (last && carry_last ? carry_last : carry[out ^ 1]) : nullptr, f, SmallPass{});
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
     out ^= 1;
   }
-  return cudaSuccess;
+  return run.error;
 }
 
 // Four passes of a small sort (key_bits of 25 to 32), one launch each.
@@ -950,6 +958,7 @@ cudaError_t small_sort(uint32_t* const keys[2], uint32_t* const vals[2], uint32_
   cudaError_t e = cudaFuncSetAttribute(k_sort_scatter<ROUNDS, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        static_cast<int>(kSmem));
   if (e != cudaSuccess) return e;
+  LaunchChain run{s};
   for (int p = 0; p < kPasses; ++p) {
     const int from = p & 1, to = from ^ 1;
     const bool last = p == kPasses - 1;
@@ -957,14 +966,14 @@ cudaError_t small_sort(uint32_t* const keys[2], uint32_t* const vals[2], uint32_
     if (p + 1 < kPasses - (last_counts ? 0 : 1)) pass.next = counts[p + 1];
     pass.next_shift = (p + 1) * kDigitBits;
     if (last && !last_counts && counts[p])
-      k_sort_hist<ROUNDS, true><<<tiles, kSortThreads, 0, s>>>(keys[from], count, p * kDigitBits, counts[p], tiles,
+      run(k_sort_hist<ROUNDS, true>, tiles, kSortThreads, 0, keys[from], count, p * kDigitBits, counts[p], tiles,
                                                                ClearRows{});
-    k_sort_scatter<ROUNDS, true><<<tiles, kSortThreads, kSmem, s>>>(
+    run(k_sort_scatter<ROUNDS, true>, tiles, kSortThreads, kSmem,
         keys[from], index_values && p == 0 ? nullptr : vals[from], last ? nullptr : keys[to], vals[to], count,
         p * kDigitBits, counts[p], tiles, carry ? carry[from] : nullptr,
         carry ? (last ? carry_last : carry[to]) : nullptr, last ? fin : FinalGather{}, pass);
   }
-  return cudaGetLastError();
+  return run.error;
 }
 
 }  // namespace
@@ -978,6 +987,7 @@ namespace {
 // --- record copy -------------------------------------------------------------------
 
 __global__ void __launch_bounds__(256) k_copy16(const uint4* __restrict__ src, uint4* __restrict__ dst, uint32_t n) {
+  after_previous();
   for (uint64_t i = blockIdx.x * 256ull + threadIdx.x; i < n; i += gridDim.x * 256ull) dst[i] = __ldcs(src + i);
 }
 
@@ -1049,25 +1059,27 @@ cudaError_t small_morton(uint4* pts, uint32_t n, bool fine, uint4* copy, uint32_
   };
   const uint32_t steps = static_cast<uint32_t>(ceil_div(n, 256 * kStreamUnroll));
   const uint32_t parts = steps < kBoundsParts ? steps : kBoundsParts;
-  k_bounds<true><<<parts, 256, 0, s>>>(pts, n, bounds, fine ? nullptr : copy);
+  LaunchChain run{s};
+  run(k_bounds<true>, parts, 256, 0, pts, n, bounds, fine ? nullptr : copy);
   if (!fine) {
     uint32_t* const counts[4] = {counts_at(vals[0], 0), counts_at(pts, 0), counts_at(pts, 1), counts_at(keys[0], 0)};
-    k_morton<ROUNDS, true><<<tiles, kSortThreads, 0, s>>>(copy, n, bounds, keys[0], counts[0], tiles, parts,
+    run(k_morton<ROUNDS, true>, tiles, kSortThreads, 0, copy, n, bounds, keys[0], counts[0], tiles, parts,
                                                          ClearRows{{counts[1], counts[2], nullptr}});
+    if (run.error != cudaSuccess) return run.error;
     return small_sort<ROUNDS>(keys, vals, n, true, counts, false, nullptr, nullptr, fin, s);
   }
   uint32_t* const free_words = hi[1] + (hi[1] - hi[0]);
   uint32_t* const low[4] = {counts_at(vals[0], 0), counts_at(free_words, 0), counts_at(free_words, 1),
                             counts_at(free_words, 2)};
-  k_morton63<ROUNDS, true><<<tiles, kSortThreads, 0, s>>>(pts, n, bounds, keys[0], hi[0], low[0], tiles, parts,
+  run(k_morton63<ROUNDS, true>, tiles, kSortThreads, 0, pts, n, bounds, keys[0], hi[0], low[0], tiles, parts,
                                                          ClearRows{{low[1], low[2], low[3]}});
-  const cudaError_t e = small_sort<ROUNDS>(keys, vals, n, true, low, true, hi, keys[0], FinalGather{}, s);
-  if (e != cudaSuccess) return e;
-  k_copy16<<<grid, 256, 0, s>>>(pts, copy, n);
+  if (run.error == cudaSuccess) run.error = small_sort<ROUNDS>(keys, vals, n, true, low, true, hi, keys[0], FinalGather{}, s);
+  run(k_copy16, grid, 256, 0, pts, copy, n);
   uint32_t* const high[4] = {counts_at(pts, 0), counts_at(pts, 1), counts_at(pts, 2), counts_at(keys[0], 0)};
   if (high[0])
-    k_sort_hist<ROUNDS, true><<<tiles, kSortThreads, 0, s>>>(keys[0], n, 0, high[0], tiles,
+    run(k_sort_hist<ROUNDS, true>, tiles, kSortThreads, 0, keys[0], n, 0, high[0], tiles,
                                                              ClearRows{{high[1], high[2], nullptr}});
+  if (run.error != cudaSuccess) return run.error;
   return small_sort<ROUNDS>(keys, vals, n, false, high, false, nullptr, nullptr, fin, s);
 }
 
@@ -1120,29 +1132,29 @@ cudaError_t launch_reorder(uint4* pts, uint32_t n, uint64_t seed, int mode, void
     case 24: return small_morton<24>(pts, n, fine, copy, keys, vals, hi, counts, fin, grid, s);
     default: break;
   }
-  k_bounds_init<<<1, 32, 0, s>>>(misc);
+  LaunchChain run{s};
+  run(k_bounds_init, 1, 32, 0, misc);
   if (!fine) {
-    k_bounds<false><<<grid, 256, 0, s>>>(pts, n, misc, copy);
-    k_morton<kSortRounds, false><<<tiles, kSortThreads, 0, s>>>(pts, n, misc, keys[0], counts, tiles, 1, ClearRows{});
-    e = radix_sort<kSortRounds>(keys, vals, n, 30, counts, partials, s, out, true, true, nullptr, nullptr, &fin);
-    if (e != cudaSuccess) return e;
-    return cudaGetLastError();
+    run(k_bounds<false>, grid, 256, 0, pts, n, misc, copy);
+    run(k_morton<kSortRounds, false>, tiles, kSortThreads, 0, pts, n, misc, keys[0], counts, tiles, 1, ClearRows{});
+    if (run.error != cudaSuccess) return run.error;
+    return radix_sort<kSortRounds>(keys, vals, n, 30, counts, partials, s, out, true, true, nullptr, nullptr, &fin);
   }
   // 63-bit code: the high halves ride along with their keys while the low
   // halves are sorted, in two buffers in the record-copy region; the last
   // pass leaves them in keys[0] (the low halves are no longer needed), which
   // frees the region for the record copy.  Then the high halves are sorted,
   // and that sort's last pass moves the records.
-  k_bounds<false><<<grid, 256, 0, s>>>(pts, n, misc, nullptr);
-  k_morton63<kSortRounds, false><<<tiles, kSortThreads, 0, s>>>(pts, n, misc, keys[0], hi[0], counts, tiles, 1, ClearRows{});
+  run(k_bounds<false>, grid, 256, 0, pts, n, misc, nullptr);
+  run(k_morton63<kSortRounds, false>, tiles, kSortThreads, 0, pts, n, misc, keys[0], hi[0], counts, tiles, 1, ClearRows{});
   int a = 0;
+  if (run.error != cudaSuccess) return run.error;
   e = radix_sort<kSortRounds>(keys, vals, n, 32, counts, partials, s, a, true, true, hi, keys[0]);
   if (e != cudaSuccess) return e;
   if (a != 0) return cudaErrorUnknown;  // 4 passes: the values are in vals[0]
-  k_copy16<<<grid, 256, 0, s>>>(pts, copy, n);
-  e = radix_sort<kSortRounds>(keys, vals, n, 31, counts, partials, s, out, false, false, nullptr, nullptr, &fin);
-  if (e != cudaSuccess) return e;
-  return cudaGetLastError();
+  run(k_copy16, grid, 256, 0, pts, copy, n);
+  if (run.error != cudaSuccess) return run.error;
+  return radix_sort<kSortRounds>(keys, vals, n, 31, counts, partials, s, out, false, false, nullptr, nullptr, &fin);
 }
 
 cudaError_t read_and_clear_reorder_error_word(uint32_t* out, cudaStream_t s) {
