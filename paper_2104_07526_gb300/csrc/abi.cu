@@ -469,8 +469,11 @@ pcr_status pcr_render_hq(pcr_ctx* ctx, float depth_factor, int variant, int clea
   const uint32_t n = static_cast<uint32_t>(ctx->n);
   const pcr::ViewParams v = view_params(ctx);
   cudaError_t e = cudaSuccess;
-  if (clear) e = pcr::launch_clear_hq(ctx->depth, ctx->rg, ctx->ba, pixels(ctx), ctx->stream, ctx->dev);
-  if (e == cudaSuccess) e = pcr::launch_hq_depth(variant, ctx->points, n, v, ctx->depth, ctx->stream, ctx->dev);
+  if (clear)
+    e = pcr::launch_hq_clear_and_depth(variant, ctx->points, n, v, ctx->depth, ctx->rg, ctx->ba, nullptr, ctx->stream,
+                                       ctx->dev);
+  else
+    e = pcr::launch_hq_depth(variant, ctx->points, n, v, ctx->depth, ctx->stream, ctx->dev);
   if (e == cudaSuccess)
     e = pcr::launch_hq_color(variant, ctx->points, n, v, depth_factor, ctx->depth, sizeof(uint32_t), ctx->rg, ctx->ba,
                              ctx->stream, ctx->dev);
@@ -492,11 +495,11 @@ pcr_status pcr_render_hq1r(pcr_ctx* ctx, float depth_factor, int variant, int cl
   const uint32_t n = static_cast<uint32_t>(ctx->n);
   const pcr::ViewParams v = view_params(ctx);
   cudaError_t e = cudaSuccess;
-  if (clear) {
-    e = pcr::launch_clear_hq(ctx->depth, ctx->rg, ctx->ba, pixels(ctx), ctx->stream, ctx->dev);
-    if (e == cudaSuccess) e = pcr::launch_fill_u64(ctx->primary, pixels(ctx), 0ull, ctx->stream, ctx->dev);
-  }
-  if (e == cudaSuccess) e = pcr::launch_hq_depth(variant, ctx->points, n, v, ctx->depth, ctx->stream, ctx->dev);
+  if (clear)
+    e = pcr::launch_hq_clear_and_depth(variant, ctx->points, n, v, ctx->depth, ctx->rg, ctx->ba, ctx->primary,
+                                       ctx->stream, ctx->dev);
+  else
+    e = pcr::launch_hq_depth(variant, ctx->points, n, v, ctx->depth, ctx->stream, ctx->dev);
   if (e == cudaSuccess)
     e = pcr::launch_hq1r_color(variant, ctx->points, n, v, depth_factor, ctx->depth, ctx->primary, ctx->rg, ctx->ba,
                                ctx->stream, ctx->dev);

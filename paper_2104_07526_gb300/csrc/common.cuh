@@ -330,7 +330,8 @@ __device__ __forceinline__ uint32_t lane_id() { return threadIdx.x & 31u; }
 
 // Start of every kernel (see launch_kernel): returns once the previous kernel
 // of the stream, and so everything before it, has finished and its writes are
-// visible; no kernel touches global memory before.  The branch, never taken,
+// visible; no kernel but
+// k_clear_sums touches global memory before.  The branch, never taken,
 // keeps the compiler from moving loads it takes for constant (of const
 // __restrict__ parameters) above the wait: past it they would be speculative.
 __device__ __forceinline__ void after_previous() {
@@ -341,5 +342,10 @@ __device__ __forceinline__ void after_previous() {
     __builtin_unreachable();
   }
 }
+
+// Lets the next kernel's blocks start once every block of this one has called
+// it: only for a next kernel that touches nothing of this one's before its own
+// after_previous().
+__device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 }  // namespace pcr

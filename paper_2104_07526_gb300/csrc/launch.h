@@ -22,8 +22,9 @@ struct Device {
 // the launch itself: a 1M-point frame of three launches 19.0 -> 12.3 us, 20k
 // points 11.9 -> 7.6, the seven launches of a 100k-point reorder 67 -> 48.
 // No kernel lets the next one start before its own end
-// (griddepcontrol.launch_dependents): waiting blocks then only stand in the
-// way (12.8, 7.6 and 50 us; a 2M-point reorder 278 against 231).
+// (griddepcontrol.launch_dependents), but for the clear of the high-quality
+// sums, which has something to do then: blocks that only wait stand in the way
+// (12.8, 7.6 and 50 us; a 2M-point reorder 278 against 231).
 template <class... P, class... A>
 cudaError_t launch_kernel(void (*kernel)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t s, A&&... args) {
   cudaLaunchAttribute attr{};
@@ -64,8 +65,12 @@ cudaError_t launch_resolve_rgb(const unsigned long long* keys, uint64_t npx, uin
                                cudaStream_t s, const Device& d);
 cudaError_t launch_render_basic(int variant, const uint4* pts, uint32_t n, const ViewParams& v,
                                 unsigned long long* keys, cudaStream_t s, const Device& d);
+// next_may_start: the next kernel launched is k_clear_sums (render.cu).
 cudaError_t launch_hq_depth(int variant, const uint4* pts, uint32_t n, const ViewParams& v, uint32_t* depth,
-                            cudaStream_t s, const Device& d);
+                            cudaStream_t s, const Device& d, bool next_may_start = false);
+cudaError_t launch_hq_clear_and_depth(int variant, const uint4* pts, uint32_t n, const ViewParams& v, uint32_t* depth,
+                                      unsigned long long* rg, unsigned long long* ba, unsigned long long* primary,
+                                      cudaStream_t s, const Device& d);
 // depth_base, depth_step: the pixels' depths and the bytes between them (4 for
 // a depth buffer, 8 for the upper words of a key buffer).
 cudaError_t launch_hq_color(int variant, const uint4* pts, uint32_t n, const ViewParams& v, float depth_factor,

@@ -1,6 +1,7 @@
 """Launches overlap the end of the kernel before them in the stream.  Back to
 back, with nothing waiting between, calls that read what the call (or the
 PyTorch kernel) just before them wrote give the results they give alone."""
+import numpy as np
 import pytest
 import torch
 
@@ -59,4 +60,41 @@ def test_back_to_back_calls_equal_calls_alone(n, order):
     for k, outs in enumerate(got):
         for i, (a, b) in enumerate(zip(alone[k % 3], outs)):
             assert torch.equal(a, b), (k, i)
+    r.close()
+
+
+@pytest.mark.parametrize("size", ((2048, 2047), (2048, 2048), (1024, 1023), (1024, 1024)))
+@pytest.mark.parametrize("n", (5_003, 2 * 1024 * 1024 - 1, 2 * 1024 * 1024))
+def test_sums_cleared_beside_the_depth_pass(oracle, size, n):
+    """High-quality frames on both sides of the limits from which the sums are
+    cleared beside the depth pass, back to back with other cameras and as a
+    replayed graph: the oracle's buffers and images."""
+    r = Renderer()
+    cloud = scenes.random_cloud(n, seed=n % 97).numpy()
+    r.upload(cloud)
+    matrices = [scenes.camera((1.5 + k, -2.0, 1.0), (0, 0, 0), (0, 0, 1), *size) for k in range(2)]
+    expect = [oracle.render_hq(cloud, m, *size, 1.01) for m in matrices]
+    images = [oracle.resolve_hq(e[1], e[2], 5) for e in expect]
+    r.view(matrices[0], *size)
+    fb, out = r.fb, []
+    for k in (0, 1, 0, 1):
+        pcr.pcr_set_matrix(r.h, matrices[k])
+        pcr.pcr_render_hq(r.h, 1.01, pcr.PCR_VARIANT_DEDUP_EARLYZ, True)
+        pcr.pcr_resolve(r.h, pcr.PCR_RESOLVE_HQ, fb["image"], 5)
+        out.append([fb[b].clone() for b in ("hq_depth", "hq_rg", "hq_ba", "image")])
+        pcr.pcr_render_hq1r(r.h, 1.01, pcr.PCR_VARIANT_EARLYZ, True)
+        pcr.pcr_resolve(r.h, pcr.PCR_RESOLVE_HQ1R, fb["image"], 5)
+        out[-1].append(fb["image"].clone())
+    pcr.pcr_capture_begin(r.h)
+    pcr.pcr_render_hq(r.h, 1.01, pcr.PCR_VARIANT_DEDUP_EARLYZ, True)
+    pcr.pcr_resolve(r.h, pcr.PCR_RESOLVE_HQ, fb["image"], 5)
+    graph = pcr.pcr_capture_end(r.h)
+    for _ in range(3):
+        pcr.pcr_graph_launch(r.h, graph)
+    out.append([fb[b].clone() for b in ("hq_depth", "hq_rg", "hq_ba", "image")])
+    torch.cuda.synchronize()
+    pcr.pcr_graph_destroy(graph)
+    for k, got in zip((0, 1, 0, 1, 1), out):
+        for a, b in zip(got, (*expect[k], images[k], images[k])):
+            assert np.array_equal(a.cpu().numpy().view(b.dtype), b), k
     r.close()
