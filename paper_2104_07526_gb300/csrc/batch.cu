@@ -230,25 +230,25 @@ __global__ void __launch_bounds__(T) k_batch_phase1(const Tables* __restrict__ t
       const BatchView& bv = sh.views[sh.order[i]];
       uint32_t pix[U];
       float w[U];
-      bool vis[U];
+      bool vis[U], group = true;
       project_all<U>(bv.vp, r, ok, pix, w, vis);
-      // every slot's early read first: one L2 round trip per view
-      bool group = true;
+      // every slot's early read first: one L2 round trip per view.  A culled
+      // slot reads 0, below every key and depth, so the early test drops it.
       if (bv.flags & PCR_BATCH_BASIC) {
         unsigned long long seen[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) seen[u] = vis[u] ? load_relaxed_u64(bv.keys + pix[u]) : 0ull;
 #pragma unroll
         for (int u = 0; u < U; ++u)
-          emit_key<PCR_VARIANT_EARLYZ>(bv.keys, vis[u], pix[u], make_key(w[u], slot_index<U, L>(base, u)), seen[u], pol_fb, group,
-                           u == 0);
+          emit_key<PCR_VARIANT_EARLYZ>(bv.keys, true, pix[u], make_key(w[u], slot_index<U, L>(base, u)), seen[u],
+                                       pol_fb, group, u == 0);
       } else {
         uint32_t seen[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) seen[u] = vis[u] ? load_relaxed_u32(bv.depth + pix[u]) : 0u;
 #pragma unroll
         for (int u = 0; u < U; ++u)
-          emit_depth<PCR_VARIANT_EARLYZ>(bv.depth, vis[u], pix[u], __float_as_uint(w[u]), seen[u], pol_fb, group, u == 0);
+          emit_depth<PCR_VARIANT_EARLYZ>(bv.depth, true, pix[u], __float_as_uint(w[u]), seen[u], pol_fb, group, u == 0);
       }
     }
   });
@@ -269,9 +269,8 @@ __global__ void __launch_bounds__(T, 1024 / T) k_batch_phase2(const Tables* __re
       const BatchView& bv = sh.views[sh.order[i]];
       uint32_t pix[U];
       float w[U];
-      bool vis[U];
+      bool vis[U], contrib[U];
       project_all<U>(bv.vp, r, ok, pix, w, vis);
-      bool contrib[U];
       contributes<U>(depth_source(bv), factor, pix, w, vis, contrib);
       emit_colors<U, true>(bv.rg, bv.ba, contrib, pix, r, pol_fb);
     }

@@ -317,19 +317,19 @@ __device__ __forceinline__ float read_depth(const DepthSource& src, uint32_t pix
 
 // Sec. 3.5 colour-pass test: a visible point contributes when
 // w <= fl(depth * factor), with the depth its pixel holds after the depth
-// pass.  The products of two slots form one paired instruction (each half
-// rounded as the scalar product).
+// pass (NaN for a culled slot, which fails).  The products of two slots form
+// one paired instruction (each half rounded as the scalar product).
 template <int U>
 __device__ __forceinline__ void contributes(const DepthSource& depth, float factor, const uint32_t (&pix)[U],
                                             const float (&w)[U], const bool (&vis)[U], bool (&contrib)[U]) {
   float d[U], thr[U];
 #pragma unroll
-  for (int u = 0; u < U; ++u) d[u] = vis[u] ? read_depth(depth, pix[u]) : 0.0f;
+  for (int u = 0; u < U; ++u) d[u] = vis[u] ? read_depth(depth, pix[u]) : __uint_as_float(0x7FC00000u);
 #pragma unroll
   for (int u = 0; u + 1 < U; u += 2) f2_unpack(f2_mul(f2_pack(d[u], d[u + 1]), f2_bcast(factor)), thr[u], thr[u + 1]);
   if constexpr (U % 2 == 1) thr[U - 1] = __fmul_rn(d[U - 1], factor);
 #pragma unroll
-  for (int u = 0; u < U; ++u) contrib[u] = vis[u] && w[u] <= thr[u];
+  for (int u = 0; u < U; ++u) contrib[u] = w[u] <= thr[u];
 }
 
 __device__ __forceinline__ uint32_t lanemask_lt() {
