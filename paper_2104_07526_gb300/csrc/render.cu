@@ -60,31 +60,33 @@ __device__ __forceinline__ void debug_check_pixels(const ViewParams& v, const ui
 #endif
 }
 
-#ifndef PCR_GEOMETRY_UNROLL
-#define PCR_GEOMETRY_UNROLL 4
-#endif
-#ifndef PCR_GEOMETRY_MIN_BLOCKS
-#define PCR_GEOMETRY_MIN_BLOCKS 1
-#endif
-
 constexpr int kThreads = 256;
-// Points per lane per chunk, and the resident blocks per SM the geometry
-// kernels are compiled for (a register cap).
-constexpr int kUnroll = PCR_GEOMETRY_UNROLL;
-constexpr int kMinBlocks = PCR_GEOMETRY_MIN_BLOCKS;
-// Each chunk runs in three phases so independent memory round trips overlap:
-// project all U points, issue all U early reads, then test and write.
-// P selects the key payload: the point index, or the 24-bit colour.  The
-// kernels are held to 40 registers (6 resident blocks of 256 threads per SM):
-// the frame is latency-bound, and one resident block fewer costs more than
-// the few instructions the register cap adds.
-constexpr int kRenderMinBlocks = kMinBlocks < 6 ? 6 : kMinBlocks;
-// The HQ depth and colour passes, HQS1R's included, take the same cap (40
-// registers each).
-constexpr int kHqMinBlocks = kMinBlocks < 6 ? 6 : kMinBlocks;
+// Points per lane per chunk.  Each chunk runs in three phases so independent
+// memory round trips overlap: project all U points, issue all U early reads,
+// then test and write.
+constexpr int kUnroll = 4;
+// The key and depth passes of clouds of up to kFewPoints points take chunks of
+// half the size: a persistent grid of 7296 warps walks few chunks of 128 points
+// each (4M points: 4.3, so a warp waits for 5), and with 32 registers two more
+// blocks fit an SM, which hides more of the reads that miss.  Key frames
+// (dedup+early-z) of 3M points 26.4 -> 23.0 us, 10M 50.7 -> 48.4, 30M
+// 103.0 -> 100.8, 50M in generation order (early-z) 274 -> 270; HQ frames 4M
+// at 4K 114.8 -> 113.3, 50M 305.7 -> 302.0.  From 100M points on the fewer
+// instructions of the larger chunk win (HQ 548 against 552 us at 100M, 800M
+// key frame 1.830 against 1.881 ms).  The colour passes join points inside a
+// lane, so they keep four.
+constexpr int kFewUnroll = 2;
+constexpr uint32_t kFewPoints = 1u << 26;
+// Resident blocks of 256 threads per SM the kernels are compiled for (a
+// register cap: 40, or 32 for the smaller chunks): the frame is latency-bound,
+// and one resident block fewer costs more than the few instructions the cap
+// adds.  The HQ colour passes take the cap of the larger chunk.
+template <int U>
+constexpr int kMinBlocksOf = U <= kFewUnroll ? 8 : 6;
+constexpr int kHqMinBlocks = kMinBlocksOf<kUnroll>;
 
 template <int V, int U, int P>
-__global__ void __launch_bounds__(kThreads, kRenderMinBlocks) k_render_basic(const uint4* __restrict__ pts, uint32_t n, ViewParams v,
+__global__ void __launch_bounds__(kThreads, kMinBlocksOf<U>) k_render_basic(const uint4* __restrict__ pts, uint32_t n, ViewParams v,
                                                            unsigned long long* __restrict__ fb) {
   after_previous();
   constexpr int L = kInterleaved;
@@ -175,7 +177,7 @@ __device__ __forceinline__ void busy_update(unsigned long long* __restrict__ fb,
 }
 
 template <int U>
-__global__ void __launch_bounds__(kThreads, kMinBlocks) k_render_busy(const uint4* __restrict__ pts, uint32_t n, ViewParams v,
+__global__ void __launch_bounds__(kThreads) k_render_busy(const uint4* __restrict__ pts, uint32_t n, ViewParams v,
                                                           unsigned long long* __restrict__ fb,
                                                           uint32_t* __restrict__ locks, uint64_t limit_ns) {
   after_previous();
@@ -204,7 +206,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) k_render_busy(const uint
 // ---------------------------------------------------------------------------
 
 template <int V, int U>
-__global__ void __launch_bounds__(kThreads, kHqMinBlocks) k_hq_depth(const uint4* __restrict__ pts, uint32_t n, ViewParams v,
+__global__ void __launch_bounds__(kThreads, kMinBlocksOf<U>) k_hq_depth(const uint4* __restrict__ pts, uint32_t n, ViewParams v,
                                                        uint32_t* __restrict__ depth, bool next_may_start) {
   after_previous();
   if (next_may_start) let_next_start();
@@ -539,11 +541,22 @@ dim3 screen_grid(uint64_t npx, const Device& d) {
 constexpr bool kCanPairLoad = kUnroll % 2 == 0;
 bool pairs_aligned(const uint4* pts) { return kCanPairLoad && (reinterpret_cast<uintptr_t>(pts) & 31u) == 0; }
 
+template <int V, int P, int U>
+cudaError_t launch_basic_u(const uint4* pts, uint32_t n, const ViewParams& v, unsigned long long* keys, cudaStream_t s,
+                           const Device& d) {
+  constexpr auto k = k_render_basic<V, U, P>;
+  return launch_kernel(k, geometry_grid<k, U>(n, d), kThreads, 0, s, pts, n, v, keys);
+}
+
 template <int V, int P>
 cudaError_t launch_basic_v(const uint4* pts, uint32_t n, const ViewParams& v, unsigned long long* keys, cudaStream_t s,
                            const Device& d) {
-  constexpr auto k = k_render_basic<V, kUnroll, P>;
-  return launch_kernel(k, geometry_grid<k, kUnroll>(n, d), kThreads, 0, s, pts, n, v, keys);
+  // pure deduplication judges a chunk by its first row and gains nothing from
+  // smaller ones (50M points 395 and 396 us)
+  if constexpr (V != PCR_VARIANT_DEDUP) {
+    if (n <= kFewPoints) return launch_basic_u<V, P, kFewUnroll>(pts, n, v, keys, s, d);
+  }
+  return launch_basic_u<V, P, kUnroll>(pts, n, v, keys, s, d);
 }
 
 template <int P>
@@ -561,11 +574,18 @@ cudaError_t launch_basic_p(int variant, const uint4* pts, uint32_t n, const View
   }
 }
 
+template <int V, int U>
+cudaError_t launch_depth_u(const uint4* pts, uint32_t n, const ViewParams& v, uint32_t* depth, cudaStream_t s,
+                           const Device& d, bool next_may_start) {
+  constexpr auto k = k_hq_depth<V, U>;
+  return launch_kernel(k, geometry_grid<k, U>(n, d), kThreads, 0, s, pts, n, v, depth, next_may_start);
+}
+
 template <int V>
 cudaError_t launch_depth_v(const uint4* pts, uint32_t n, const ViewParams& v, uint32_t* depth, cudaStream_t s,
                            const Device& d, bool next_may_start) {
-  constexpr auto k = k_hq_depth<V, kUnroll>;
-  return launch_kernel(k, geometry_grid<k, kUnroll>(n, d), kThreads, 0, s, pts, n, v, depth, next_may_start);
+  if (n <= kFewPoints) return launch_depth_u<V, kFewUnroll>(pts, n, v, depth, s, d, next_may_start);
+  return launch_depth_u<V, kUnroll>(pts, n, v, depth, s, d, next_may_start);
 }
 
 }  // namespace
@@ -672,12 +692,18 @@ cudaError_t launch_hq_color(int variant, const uint4* pts, uint32_t n, const Vie
 template <int P>
 void prewarm_basic(const Device& d) {
   geometry_grid<k_render_basic<PCR_VARIANT_ATOMICMIN, kUnroll, P>, kUnroll>(1, d);
+  geometry_grid<k_render_basic<PCR_VARIANT_ATOMICMIN, kFewUnroll, P>, kFewUnroll>(1, d);
   geometry_grid<k_render_basic<PCR_VARIANT_EARLYZ, kUnroll, P>, kUnroll>(1, d);
+  geometry_grid<k_render_basic<PCR_VARIANT_EARLYZ, kFewUnroll, P>, kFewUnroll>(1, d);
   geometry_grid<k_render_basic<PCR_VARIANT_DEDUP, kUnroll, P>, kUnroll>(1, d);
   geometry_grid<k_render_basic<PCR_VARIANT_DEDUP_EARLYZ, kUnroll, P>, kUnroll>(1, d);
+  geometry_grid<k_render_basic<PCR_VARIANT_DEDUP_EARLYZ, kFewUnroll, P>, kFewUnroll>(1, d);
   geometry_grid<k_render_basic<PCR_VARIANT_REDUCE, kUnroll, P>, kUnroll>(1, d);
+  geometry_grid<k_render_basic<PCR_VARIANT_REDUCE, kFewUnroll, P>, kFewUnroll>(1, d);
   geometry_grid<k_render_basic<PCR_VARIANT_REDUCE_EARLYZ, kUnroll, P>, kUnroll>(1, d);
+  geometry_grid<k_render_basic<PCR_VARIANT_REDUCE_EARLYZ, kFewUnroll, P>, kFewUnroll>(1, d);
   geometry_grid<k_render_basic<PCR_VARIANT_JUST_SET, kUnroll, P>, kUnroll>(1, d);
+  geometry_grid<k_render_basic<PCR_VARIANT_JUST_SET, kFewUnroll, P>, kFewUnroll>(1, d);
 }
 
 // Every single-view geometry kernel's occupancy query (cached per kernel):
@@ -687,9 +713,13 @@ void prewarm_single_view(const Device& d) {
   prewarm_basic<kPayloadRgb>(d);
   geometry_grid<k_render_busy<kUnroll>, kUnroll>(1, d);
   geometry_grid<k_hq_depth<PCR_VARIANT_ATOMICMIN, kUnroll>, kUnroll>(1, d);
+  geometry_grid<k_hq_depth<PCR_VARIANT_ATOMICMIN, kFewUnroll>, kFewUnroll>(1, d);
   geometry_grid<k_hq_depth<PCR_VARIANT_EARLYZ, kUnroll>, kUnroll>(1, d);
+  geometry_grid<k_hq_depth<PCR_VARIANT_EARLYZ, kFewUnroll>, kFewUnroll>(1, d);
   geometry_grid<k_hq_depth<PCR_VARIANT_DEDUP, kUnroll>, kUnroll>(1, d);
+  geometry_grid<k_hq_depth<PCR_VARIANT_DEDUP, kFewUnroll>, kFewUnroll>(1, d);
   geometry_grid<k_hq_depth<PCR_VARIANT_DEDUP_EARLYZ, kUnroll>, kUnroll>(1, d);
+  geometry_grid<k_hq_depth<PCR_VARIANT_DEDUP_EARLYZ, kFewUnroll>, kFewUnroll>(1, d);
   geometry_grid<k_hq_color<false, kUnroll, false>, kUnroll>(1, d);
   geometry_grid<k_hq_color<true, kUnroll, kCanPairLoad>, kUnroll>(1, d);
   geometry_grid<k_hq_color<true, kUnroll, false>, kUnroll>(1, d);
