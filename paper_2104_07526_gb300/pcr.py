@@ -194,6 +194,8 @@ def load_library(path: str) -> C.CDLL:
 def lib() -> C.CDLL:
     """Load libpcr.so (raises if it has not been built)."""
     global _lib
+    if _lib is not None:  # loaded once, never replaced by None: no lock on the way of every call
+        return _lib
     with _lock:
         if _lib is None:
             _lib = load_library(LIB_PATH)
