@@ -162,8 +162,15 @@ static_assert(kSortRounds % kMortonUnroll == 0, "whole rounds of records per til
 // are also copied there (the source the sort's last pass moves them from),
 // saving a pass.  SMALL: block b writes its own bounds to misc[6 b .. 6 b + 5]
 // (k_morton joins them) instead of joining them in misc[0 .. 5].
+// A stream of 16 bytes a point, 32 with the copy.  Large clouds take
+// kBoundsBlocks blocks per SM, two full waves of the five that its registers
+// let an SM hold: with 8, the last wave held three, and an 800M reorder took
+// 25.42 ms against 25.14 (all in one wave: 25.23).  A block joins its warps'
+// bounds before the atomics on the six shared words: one set of atomics per
+// warp held a 3M reorder at 233 us and a 10M one at 466, now 200 and 441.
+constexpr unsigned kBoundsBlocks = 10;
 template <bool SMALL>
-__global__ void __launch_bounds__(256) k_bounds(const uint4* __restrict__ pts, uint32_t n, uint32_t* misc,
+__global__ void __launch_bounds__(256, 5) k_bounds(const uint4* __restrict__ pts, uint32_t n, uint32_t* misc,
                                                 uint4* __restrict__ copy) {
   after_previous();
   uint32_t lo[3] = {0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu};
@@ -198,30 +205,26 @@ __global__ void __launch_bounds__(256) k_bounds(const uint4* __restrict__ pts, u
     lo[a] = __reduce_min_sync(kFullMask, lo[a]);
     hi[a] = __reduce_max_sync(kFullMask, hi[a]);
   }
-  if constexpr (SMALL) {
-    __shared__ uint32_t s_bounds[8][kBoundsValues];
-    if (lane_id() == 0) {
-#pragma unroll
-      for (int a = 0; a < 3; ++a) {
-        // no value: the identities k_bounds_init starts from
-        s_bounds[threadIdx.x >> 5][a] = min(lo[a], 0xFF800000u);
-        s_bounds[threadIdx.x >> 5][3 + a] = max(hi[a], 0x007FFFFFu);
-      }
-    }
-    __syncthreads();
-    if (threadIdx.x < kBoundsValues) {
-      uint32_t v = s_bounds[0][threadIdx.x];
-      for (int w = 1; w < 8; ++w)
-        v = threadIdx.x < 3 ? min(v, s_bounds[w][threadIdx.x]) : max(v, s_bounds[w][threadIdx.x]);
-      misc[kBoundsValues * blockIdx.x + threadIdx.x] = v;
-    }
-    return;
-  }
+  __shared__ uint32_t s_bounds[8][kBoundsValues];
   if (lane_id() == 0) {
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-      if (lo[a] != 0xFFFFFFFFu) atomicMin(misc + a, lo[a]);
-      if (hi[a] != 0u) atomicMax(misc + 3 + a, hi[a]);
+      // no value: the identities k_bounds_init starts from
+      s_bounds[threadIdx.x >> 5][a] = min(lo[a], 0xFF800000u);
+      s_bounds[threadIdx.x >> 5][3 + a] = max(hi[a], 0x007FFFFFu);
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x < kBoundsValues) {
+    uint32_t v = s_bounds[0][threadIdx.x];
+    for (int w = 1; w < 8; ++w)
+      v = threadIdx.x < 3 ? min(v, s_bounds[w][threadIdx.x]) : max(v, s_bounds[w][threadIdx.x]);
+    if constexpr (SMALL) {
+      misc[kBoundsValues * blockIdx.x + threadIdx.x] = v;
+    } else if (threadIdx.x < 3) {
+      atomicMin(misc + threadIdx.x, v);
+    } else {
+      atomicMax(misc + threadIdx.x, v);
     }
   }
 }
@@ -1004,9 +1007,9 @@ __global__ void __launch_bounds__(256) k_copy16(const uint4* __restrict__ src, u
   for (uint64_t i = blockIdx.x * 256ull + threadIdx.x; i < n; i += gridDim.x * 256ull) dst[i] = __ldcs(src + i);
 }
 
-unsigned stream_grid(uint64_t count, const Device& d) {
+unsigned stream_grid(uint64_t count, const Device& d, unsigned blocks_per_sm = 8) {
   const uint64_t need = ceil_div(count, 256);
-  const uint64_t cap = static_cast<uint64_t>(d.num_sms) * 8;
+  const uint64_t cap = static_cast<uint64_t>(d.num_sms) * blocks_per_sm;
   return static_cast<unsigned>(need < cap ? (need > 0 ? need : 1) : cap);
 }
 
@@ -1110,6 +1113,7 @@ cudaError_t launch_reorder(uint4* pts, uint32_t n, uint64_t seed, int mode, void
   uint32_t* partials = reinterpret_cast<uint32_t*>(ws + l.partials);
   uint32_t* misc = reinterpret_cast<uint32_t*>(ws + l.misc);
   const unsigned grid = stream_grid(n, d);
+  const unsigned bounds_grid = stream_grid(n, d, kBoundsBlocks);
   const uint32_t tiles = static_cast<uint32_t>(ceil_div(n, kTile));  // the sort's tiles
   cudaError_t e = cudaSuccess;
   int out = 0;
@@ -1148,7 +1152,7 @@ cudaError_t launch_reorder(uint4* pts, uint32_t n, uint64_t seed, int mode, void
   LaunchChain run{s};
   run(k_bounds_init, 1, 32, 0, misc);
   if (!fine) {
-    run(k_bounds<false>, grid, 256, 0, pts, n, misc, copy);
+    run(k_bounds<false>, bounds_grid, 256, 0, pts, n, misc, copy);
     run(k_morton<kSortRounds, false>, tiles, kSortThreads, 0, pts, n, misc, keys[0], counts, tiles, 1, ClearRows{});
     if (run.error != cudaSuccess) return run.error;
     return radix_sort<kSortRounds>(keys, vals, n, 30, counts, partials, s, out, true, true, nullptr, nullptr, &fin);
@@ -1158,7 +1162,7 @@ cudaError_t launch_reorder(uint4* pts, uint32_t n, uint64_t seed, int mode, void
   // pass leaves them in keys[0] (the low halves are no longer needed), which
   // frees the region for the record copy.  Then the high halves are sorted,
   // and that sort's last pass moves the records.
-  run(k_bounds<false>, grid, 256, 0, pts, n, misc, nullptr);
+  run(k_bounds<false>, bounds_grid, 256, 0, pts, n, misc, nullptr);
   run(k_morton63<kSortRounds, false>, tiles, kSortThreads, 0, pts, n, misc, keys[0], hi[0], counts, tiles, 1, ClearRows{});
   int a = 0;
   if (run.error != cudaSuccess) return run.error;

@@ -177,3 +177,24 @@ def test_small_reorder_of_points_without_bounds(r, oracle):
             expect = oracle.reorder(cloud, 3, mode)
             dev = torch.from_numpy(cloud.copy()).cuda()
             assert np.array_equal(reorder_gpu(r.h, dev, 3, mode), expect), (spoil, mode)
+
+
+@pytest.mark.parametrize("spoil", ["all", "axis", "inf", "one"])
+def test_large_reorder_of_points_without_bounds(r, oracle, spoil):
+    """As above with the bounds that blocks join by atomics; "one": a single
+    point has an extreme, in the last record."""
+    n = 384 * 6144 + 261
+    cloud = scenes.random_cloud(n, seed=2).numpy()
+    if spoil == "all":
+        cloud[:, :3] = np.float32(np.nan).view(np.int32)
+    elif spoil == "axis":
+        cloud[:, 1] = np.float32(np.nan).view(np.int32)
+    elif spoil == "inf":
+        cloud[::7, 0] = np.float32(np.inf).view(np.int32)
+        cloud[3::7, 2] = np.float32(-np.inf).view(np.int32)
+    else:
+        cloud[-1, :3] = np.array([900.0, -700.0, 800.0], np.float32).view(np.int32)
+    for mode in (pcr.PCR_ORDER_MORTON, pcr.PCR_ORDER_MORTON63):
+        expect = oracle.reorder(cloud, 3, mode)
+        dev = torch.from_numpy(cloud.copy()).cuda()
+        assert np.array_equal(reorder_gpu(r.h, dev, 3, mode), expect), mode
