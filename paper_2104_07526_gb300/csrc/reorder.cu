@@ -83,16 +83,15 @@ constexpr uint64_t ceil_div(uint64_t a, uint64_t b) { return (a + b - 1) / b; }
 // Small clouds.  Their sorts are bound by launches and by blocks too few to
 // fill the GPU, so a pass is one launch of smaller tiles: every scatter block
 // sums the counts of the tiles before its own, and counts the next pass's
-// digits as it writes (one global atomic per key).  Morton order, one launch
-// per pass against five on tiles of 6144: 60k points 136 -> 51 us, 130k
-// 149 -> 62, 390k 150 -> 81, 780k 174 -> 111, 1.5M 221 -> 170, 2.2M
-// 254 -> 240; shuffled Morton of 100k 253 -> 66 us (bound by the chain of
-// launches: seven, of about 6 us each).  Past the last limit the sums over
-// tiles cost more than a scan (3.1M: 345 against 300 us with 512 tiles); 12
-// keys per lane take over from 4 where their sums are shorter (190k points:
-// 70 against 75 us).  Keys per lane of a small sort's tiles; 0: not small.
+// digits as it writes (one global atomic per key).  Morton order, five
+// launches per pass on tiles of 6144 against one: 100k points 88 -> 42 us,
+// 200k 90 -> 54, 400k 91 -> 64, 600k 93 -> 86, 786k 92 -> 90.  Past the last
+// limit the sums over tiles cost more than a scan: 24 keys per lane took 119 us
+// against 116 at 1M points and 205 against 150 at 2.36M.  12 keys per lane take
+// over from 4 where their sums are shorter (200k points: 54 against 62 us).
+// Keys per lane of a small sort's tiles; 0: not small.
 constexpr int small_rounds(uint64_t n) {
-  return n <= 128 * kTileOf<4> ? 4 : n <= 256 * kTileOf<12> ? 12 : n <= 384 * kTileOf<24> ? 24 : 0;
+  return n <= 128 * kTileOf<4> ? 4 : n <= 256 * kTileOf<12> ? 12 : 0;
 }
 constexpr uint32_t kSumUnroll = 32;   // counts of other tiles in flight per thread (16: 74 us, 32: 66 at 100k)
 constexpr uint32_t kBoundsParts = 128;  // blocks of a small cloud's k_bounds, at most
@@ -1146,7 +1145,6 @@ cudaError_t launch_reorder(uint4* pts, uint32_t n, uint64_t seed, int mode, void
   switch (small_rounds(n)) {
     case 4: return small_morton<4>(pts, n, fine, copy, keys, vals, hi, counts, fin, grid, s);
     case 12: return small_morton<12>(pts, n, fine, copy, keys, vals, hi, counts, fin, grid, s);
-    case 24: return small_morton<24>(pts, n, fine, copy, keys, vals, hi, counts, fin, grid, s);
     default: break;
   }
   LaunchChain run{s};
