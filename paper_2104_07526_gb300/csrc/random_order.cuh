@@ -445,6 +445,10 @@ cudaError_t random_order(uint4* pts, uint4* copy, uint32_t n, uint64_t seed, uin
                          uint32_t* counters, uint32_t* partials, RandomOut out, cudaStream_t s, const Device& d) {
   const RandomSplit p = random_split(n);
   LaunchChain run{s};
+  // The limit belongs to the kernel, for every stream and host thread: always
+  // the most any size asks for.  A limit per call (98 to 115 KB by the digits)
+  // could be lowered by another thread's call before this one's launch, which
+  // then fails.  How many blocks an SM holds follows from what a launch asks for.
   auto allow = [&](auto kernel, size_t bytes) {
     if (run.error == cudaSuccess)
       run.error = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
@@ -462,7 +466,7 @@ cudaError_t random_order(uint4* pts, uint4* copy, uint32_t n, uint64_t seed, uin
     run(k_random_count_first, blocks, kPartThreads, sizeof(uint32_t) * radix, n, seed, p.buckets, p.second, radix,
                                                                                first);
     run(k_scan_partials, 1, 1024, 0, first, radix);
-    allow(k_random_partition<REC, true>, partition_smem<REC>(radix));
+    allow(k_random_partition<REC, true>, partition_smem<REC>(1u << kMaxPassBits));
     run(k_random_partition<REC, true>, tiles, kPartThreads, partition_smem<REC>(radix), pts, nullptr, copy, idx[0], n, seed, p.buckets, p.second, radix, first);
     rin = copy;
     iin = idx[0];
@@ -474,7 +478,7 @@ cudaError_t random_order(uint4* pts, uint4* copy, uint32_t n, uint64_t seed, uin
       run(k_random_count_second, chunks, kPartThreads, sizeof(uint32_t) * low, idx[0], n, seed, p.buckets, p.second,
                                                                                 both);
       if (run.error == cudaSuccess) run.error = exclusive_scan(both, p.buckets, partials, s);
-      allow(k_random_partition<REC, false>, partition_smem<REC>(low));
+      allow(k_random_partition<REC, false>, partition_smem<REC>(1u << kMaxPassBits));
       run(k_random_partition<REC, false>, tiles, kPartThreads, partition_smem<REC>(low), copy, idx[0], pts, idx[1], n, seed, p.buckets, p.second, low, both);
       rin = pts;
       iin = idx[1];
