@@ -303,7 +303,11 @@ PCR_API pcr_status pcr_reorder_workspace_size(uint64_t n, uint64_t *bytes);
  * nor the workspace; the call may also use it as scratch before it writes
  * the result), receives perm[new] = old.
  * Errors: PCR_ERR_ARG for a bad mode, pointer or n; PCR_ERR_WORKSPACE if
- * workspace_bytes is too small or the workspace is NULL. */
+ * workspace_bytes is too small or the workspace is NULL; PCR_ERR_CUDA if a
+ * launch fails.  After a failed launch the points of the Morton orders are as
+ * they were (their last launch is the only one that writes them), those of
+ * PCR_ORDER_SHUFFLE the same records in some order; the workspace and
+ * dev_perm_out hold nothing of use. */
 PCR_API pcr_status pcr_reorder_morton_shuffle128(pcr_ctx *ctx, void *dev_points, uint64_t n, uint64_t seed, int mode,
                                          void *dev_workspace, uint64_t workspace_bytes, uint32_t *dev_perm_out);
 
@@ -693,6 +697,13 @@ PCR_API const char *pcr_status_string(pcr_status status);
  * PCR_ERR_UNSUPPORTED in release builds; PCR_ERR_ARG for NULL arguments;
  * PCR_ERR_CUDA if the copy fails. */
 PCR_API pcr_status pcr_debug_counters(pcr_ctx *ctx, uint64_t out[4]);
+
+/* Debug builds only: kernel launch number `after` from now (0: the next) of
+ * the calling host thread fails, once, on the host: the kernel is not
+ * launched, and the call that wanted it reports the error.  A negative
+ * `after` cancels it.  It shows what a call that fails half-way leaves
+ * behind.  Errors: PCR_ERR_UNSUPPORTED in release builds. */
+PCR_API pcr_status pcr_debug_fail_launch(int after);
 
 /* Read and clear the device-side error word of the context's device
  * (synchronises the stream): PCR_DEVICE_ERROR_KEY_RANGE when a resolve found

@@ -803,6 +803,16 @@ pcr_status pcr_debug_counters(pcr_ctx* ctx, uint64_t out[4]) {
   return from_cuda(e);
 }
 
+pcr_status pcr_debug_fail_launch(int after) {
+#ifdef PCR_DEBUG
+  pcr::debug_launches_left = after;
+  return PCR_OK;
+#else
+  (void)after;
+  return PCR_ERR_UNSUPPORTED;
+#endif
+}
+
 pcr_status pcr_last_device_error(pcr_ctx* ctx, uint32_t* code) {
   if (!ctx || ctx->capture || !code) return PCR_ERR_ARG;
   DeviceScope scope(ctx->dev.id);

@@ -16,6 +16,11 @@ struct Device {
   int num_sms = 0;
 };
 
+#ifdef PCR_DEBUG
+// Launches this host thread makes before one fails (pcr_debug_fail_launch); none does below 0.
+inline thread_local int debug_launches_left = -1;
+#endif
+
 // Launch a kernel whose blocks may start as the blocks of the stream's previous
 // kernel end.  Every kernel launched so begins with after_previous() in every
 // thread, so its work starts where a plain launch's would; what overlaps is
@@ -27,6 +32,9 @@ struct Device {
 // (12.8, 7.6 and 50 us; a 2M-point reorder 278 against 231).
 template <class... P, class... A>
 cudaError_t launch_kernel(void (*kernel)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t s, A&&... args) {
+#ifdef PCR_DEBUG
+  if (debug_launches_left >= 0 && debug_launches_left-- == 0) return cudaErrorLaunchOutOfResources;
+#endif
   cudaLaunchAttribute attr{};
   attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr.val.programmaticStreamSerializationAllowed = 1;

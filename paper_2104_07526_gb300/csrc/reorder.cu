@@ -160,7 +160,8 @@ static_assert(kSortRounds % kMortonUnroll == 0, "whole rounds of records per til
 // codes do not depend on the sign of a zero bound).  With `copy`, the records
 // are also copied there (the source the sort's last pass moves them from),
 // saving a pass.  SMALL: block b writes its own bounds to misc[6 b .. 6 b + 5]
-// (k_morton joins them) instead of joining them in misc[0 .. 5].
+// (k_morton joins them) instead of joining them in misc[0 .. 5], and the first
+// copy_from records are left to a later kernel.
 // A stream of 16 bytes a point, 32 with the copy.  Large clouds take
 // kBoundsBlocks blocks per SM, two full waves of the five that its registers
 // let an SM hold: with 8, the last wave held three, and an 800M reorder took
@@ -170,7 +171,7 @@ static_assert(kSortRounds % kMortonUnroll == 0, "whole rounds of records per til
 constexpr unsigned kBoundsBlocks = 10;
 template <bool SMALL>
 __global__ void __launch_bounds__(256, 5) k_bounds(const uint4* __restrict__ pts, uint32_t n, uint32_t* misc,
-                                                uint4* __restrict__ copy) {
+                                                uint4* __restrict__ copy, uint32_t copy_from) {
   after_previous();
   uint32_t lo[3] = {0xFFFFFFFFu, 0xFFFFFFFFu, 0xFFFFFFFFu};
   uint32_t hi[3] = {0u, 0u, 0u};
@@ -187,7 +188,7 @@ __global__ void __launch_bounds__(256, 5) k_bounds(const uint4* __restrict__ pts
     for (int u = 0; u < kStreamUnroll; ++u) {
       const uint64_t i = i0 + 256ull * u;
       if (i >= n) break;
-      if (copy) __stcs(copy + i, r[u]);
+      if (copy && (!SMALL || i >= copy_from)) __stcs(copy + i, r[u]);
       const float v[3] = {__uint_as_float(r[u].x), __uint_as_float(r[u].y), __uint_as_float(r[u].z)};
 #pragma unroll
       for (int a = 0; a < 3; ++a) {
@@ -270,6 +271,46 @@ __device__ __forceinline__ void clear_rows(const ClearRows& rows) {
   for (int k = 0; k < 3; ++k)
     if (rows.at[k]) rows.at[k][blockIdx.x * kRadix + threadIdx.x] = 0u;
 }
+
+// Records a kernel with one block per tile copies, `per_tile` for each, those
+// from 0 on (src null: none).
+struct CopyRecords {
+  const uint4* src = nullptr;
+  uint4* dst = nullptr;
+  uint32_t per_tile = 0;
+};
+
+// The block's part of a CopyRecords: load() before the kernel's own work takes
+// kStreamUnroll records per thread, finish() after it stores them and copies
+// the rest (of a small cloud: 32-bit positions do not overflow).
+struct BlockCopy {
+  const CopyRecords& c;
+  uint32_t at, end;
+  uint4 r[kStreamUnroll];
+
+  __device__ __forceinline__ BlockCopy(const CopyRecords& copy, uint32_t n) : c(copy) {
+    at = blockIdx.x * c.per_tile + threadIdx.x;
+    end = c.src ? min((blockIdx.x + 1) * c.per_tile, n) : 0u;
+  }
+  __device__ __forceinline__ void load() {
+#pragma unroll
+    for (uint32_t u = 0; u < kStreamUnroll; ++u)
+      if (at + kSortThreads * u < end) r[u] = __ldcs(c.src + at + kSortThreads * u);
+  }
+  __device__ __forceinline__ void store() {
+#pragma unroll
+    for (uint32_t u = 0; u < kStreamUnroll; ++u)
+      if (at + kSortThreads * u < end) c.dst[at + kSortThreads * u] = r[u];
+    at += kSortThreads * kStreamUnroll;
+  }
+  __device__ __forceinline__ void finish() {
+    store();
+    while (at < end) {
+      load();
+      store();
+    }
+  }
+};
 
 template <int ROUNDS, bool SMALL>
 __device__ __forceinline__ void count_tile_digits(TileKeys<ROUNDS>& sh, uint32_t valid, uint32_t* __restrict__ counts,
@@ -502,9 +543,13 @@ __device__ __forceinline__ uint32_t digit_peers(uint32_t d, uint32_t valid) {
 template <int ROUNDS, bool SMALL>
 __global__ void __launch_bounds__(kSortThreads) k_sort_hist(const uint32_t* __restrict__ keys, uint32_t n, int shift,
                                                             uint32_t* __restrict__ counts, uint32_t tiles,
-                                                            ClearRows zero) {
+                                                            ClearRows zero, CopyRecords copy) {
   after_previous();
-  if constexpr (SMALL) clear_rows(zero);
+  BlockCopy records(copy, n);
+  if constexpr (SMALL) {
+    records.load();
+    clear_rows(zero);
+  }
   __shared__ uint32_t hist[kSortWarps][kRadix];
 #pragma unroll
   for (int w = 0; w < kSortWarps; ++w) hist[w][threadIdx.x] = 0;
@@ -543,8 +588,12 @@ __global__ void __launch_bounds__(kSortThreads) k_sort_hist(const uint32_t* __re
   uint32_t c = 0;
 #pragma unroll
   for (int w = 0; w < kSortWarps; ++w) c += hist[w][threadIdx.x];
-  if constexpr (SMALL) counts[blockIdx.x * kRadix + threadIdx.x] = c;
-  else counts[static_cast<uint64_t>(threadIdx.x) * tiles + blockIdx.x] = c;
+  if constexpr (SMALL) {
+    counts[blockIdx.x * kRadix + threadIdx.x] = c;
+    records.finish();
+  } else {
+    counts[static_cast<uint64_t>(threadIdx.x) * tiles + blockIdx.x] = c;
+  }
 }
 
 template <int NT>
@@ -946,7 +995,7 @@ cudaError_t radix_sort(uint32_t* keys[2], uint32_t* vals[2], uint32_t count, int
   LaunchChain run{s};
   for (int shift = 0; shift < key_bits; shift += kDigitBits) {
     const bool last = shift + kDigitBits >= key_bits;
-    if (!(first_counted && shift == 0)) run(k_sort_hist<ROUNDS, false>, tiles, kSortThreads, 0, keys[out], count, shift, counts, tiles, ClearRows{});
+    if (!(first_counted && shift == 0)) run(k_sort_hist<ROUNDS, false>, tiles, kSortThreads, 0, keys[out], count, shift, counts, tiles, ClearRows{}, CopyRecords{});
     if (run.error == cudaSuccess) run.error = exclusive_scan(counts, static_cast<uint64_t>(kRadix) * tiles, partials, s);
     const uint32_t* vin = (index_values && shift == 0) ? nullptr : vals[out];
     uint32_t* kout = last ? nullptr : keys[out ^ 1];
@@ -962,11 +1011,12 @@ cudaError_t radix_sort(uint32_t* keys[2], uint32_t* vals[2], uint32_t count, int
 // Four passes of a small sort (key_bits of 25 to 32), one launch each.
 // counts[p] (null for a single tile) holds or receives pass p's counts: the
 // first ones are made, the next two clear; `last_counts` says that the last
-// ones are too, otherwise k_sort_hist makes them.
+// ones are too, otherwise k_sort_hist makes them, and copies what `copy` says
+// for the last pass to move.
 template <int ROUNDS>
 cudaError_t small_sort(uint32_t* const keys[2], uint32_t* const vals[2], uint32_t count, bool index_values,
                        uint32_t* const counts[4], bool last_counts, uint32_t* const* carry, uint32_t* carry_last,
-                       const FinalGather& fin, cudaStream_t s) {
+                       const FinalGather& fin, const CopyRecords& copy, cudaStream_t s) {
   constexpr int kPasses = 4;
   const uint32_t tiles = static_cast<uint32_t>(ceil_div(count, kTileOf<ROUNDS>));
   constexpr size_t kSmem = scatter_smem<ROUNDS>();
@@ -982,7 +1032,7 @@ cudaError_t small_sort(uint32_t* const keys[2], uint32_t* const vals[2], uint32_
     pass.next_shift = (p + 1) * kDigitBits;
     if (last && !last_counts && counts[p])
       run(k_sort_hist<ROUNDS, true>, tiles, kSortThreads, 0, keys[from], count, p * kDigitBits, counts[p], tiles,
-                                                               ClearRows{});
+          ClearRows{}, copy);
     run(k_sort_scatter<ROUNDS, true>, tiles, kSortThreads, kSmem,
         keys[from], index_values && p == 0 ? nullptr : vals[from], last ? nullptr : keys[to], vals[to], count,
         p * kDigitBits, counts[p], tiles, carry ? carry[from] : nullptr,
@@ -1055,14 +1105,20 @@ uint64_t reorder_workspace_bytes(uint64_t n) { return layout(n).total; }
 namespace {
 
 // Morton orders of a small cloud: bounds, codes and one launch per sort pass.
-// The counts of its passes lie in buffers that are free while they are needed:
-//   30-bit: pass 0 in vals[0]; passes 1 and 2 in the points (read from their
-//     copy from the codes on), pass 3 in keys[0];
+// The points are only read until the last pass, which moves them from their
+// copy, so a launch that fails before it leaves them as they were.  The counts
+// of the passes lie in buffers that are free while they are needed:
+//   30-bit: pass 0 in vals[0]; passes 1 and 2 at the start of the copy, whose
+//     records there follow (the others are copied by k_bounds) as the counts of
+//     pass 3 are made in keys[0];
 //   63-bit: pass 0 in vals[0], 1 to 3 behind the high halves in the copy
-//     region, 4 to 6 in the points (copied by then), 7 in keys[0].
+//     region, 4 to 6 at its start (the high halves are in keys[0] by then); the
+//     records follow as the counts of pass 7 are made in keys[0].
 // A tile of 1024 keys or more has 1 KB of counts, so a set takes at most 2 n
 // bytes (n with a full last tile): two fit a 4-byte buffer, and three fit
-// behind two of them in the copy's 16 n.  A single tile has no counts.
+// behind two of them in the copy's 16 n.  A single tile has no counts; its
+// records are copied by k_bounds (30-bit) or k_copy16.
+constexpr uint32_t kCountRecords = 2 * kRadix * sizeof(uint32_t) / sizeof(uint4);  // under two sets' counts of a tile
 template <int ROUNDS>
 cudaError_t small_morton(uint4* pts, uint32_t n, bool fine, uint4* copy, uint32_t* const keys[2],
                          uint32_t* const vals[2], uint32_t* const hi[2], uint32_t* bounds, const FinalGather& fin,
@@ -1075,27 +1131,30 @@ cudaError_t small_morton(uint4* pts, uint32_t n, bool fine, uint4* copy, uint32_
   const uint32_t steps = static_cast<uint32_t>(ceil_div(n, 256 * kStreamUnroll));
   const uint32_t parts = steps < kBoundsParts ? steps : kBoundsParts;
   LaunchChain run{s};
-  run(k_bounds<true>, parts, 256, 0, pts, n, bounds, fine ? nullptr : copy);
+  run(k_bounds<true>, parts, 256, 0, pts, n, bounds, fine ? nullptr : copy, tiles > 1 ? tiles * kCountRecords : 0u);
   if (!fine) {
-    uint32_t* const counts[4] = {counts_at(vals[0], 0), counts_at(pts, 0), counts_at(pts, 1), counts_at(keys[0], 0)};
-    run(k_morton<ROUNDS, true>, tiles, kSortThreads, 0, copy, n, bounds, keys[0], counts[0], tiles, parts,
-                                                         ClearRows{{counts[1], counts[2], nullptr}});
+    uint32_t* const counts[4] = {counts_at(vals[0], 0), counts_at(copy, 0), counts_at(copy, 1), counts_at(keys[0], 0)};
+    run(k_morton<ROUNDS, true>, tiles, kSortThreads, 0, pts, n, bounds, keys[0], counts[0], tiles, parts,
+        ClearRows{{counts[1], counts[2], nullptr}});
     if (run.error != cudaSuccess) return run.error;
-    return small_sort<ROUNDS>(keys, vals, n, true, counts, false, nullptr, nullptr, fin, s);
+    return small_sort<ROUNDS>(keys, vals, n, true, counts, false, nullptr, nullptr, fin,
+                              CopyRecords{pts, copy, kCountRecords}, s);
   }
   uint32_t* const free_words = hi[1] + (hi[1] - hi[0]);
   uint32_t* const low[4] = {counts_at(vals[0], 0), counts_at(free_words, 0), counts_at(free_words, 1),
                             counts_at(free_words, 2)};
   run(k_morton63<ROUNDS, true>, tiles, kSortThreads, 0, pts, n, bounds, keys[0], hi[0], low[0], tiles, parts,
-                                                         ClearRows{{low[1], low[2], low[3]}});
-  if (run.error == cudaSuccess) run.error = small_sort<ROUNDS>(keys, vals, n, true, low, true, hi, keys[0], FinalGather{}, s);
-  run(k_copy16, grid, 256, 0, pts, copy, n);
-  uint32_t* const high[4] = {counts_at(pts, 0), counts_at(pts, 1), counts_at(pts, 2), counts_at(keys[0], 0)};
-  if (high[0])
+      ClearRows{{low[1], low[2], low[3]}});
+  if (run.error == cudaSuccess) run.error = small_sort<ROUNDS>(keys, vals, n, true, low, true, hi, keys[0], FinalGather{}, CopyRecords{}, s);
+  uint32_t* const high[4] = {counts_at(copy, 0), counts_at(copy, 1), counts_at(copy, 2), counts_at(keys[0], 0)};
+  if (tiles > 1)
     run(k_sort_hist<ROUNDS, true>, tiles, kSortThreads, 0, keys[0], n, 0, high[0], tiles,
-                                                             ClearRows{{high[1], high[2], nullptr}});
+        ClearRows{{high[1], high[2], nullptr}}, CopyRecords{});
+  else
+    run(k_copy16, grid, 256, 0, pts, copy, n);
   if (run.error != cudaSuccess) return run.error;
-  return small_sort<ROUNDS>(keys, vals, n, false, high, false, nullptr, nullptr, fin, s);
+  return small_sort<ROUNDS>(keys, vals, n, false, high, false, nullptr, nullptr, fin,
+                            CopyRecords{pts, copy, kTileOf<ROUNDS>}, s);
 }
 
 }  // namespace
@@ -1150,7 +1209,7 @@ cudaError_t launch_reorder(uint4* pts, uint32_t n, uint64_t seed, int mode, void
   LaunchChain run{s};
   run(k_bounds_init, 1, 32, 0, misc);
   if (!fine) {
-    run(k_bounds<false>, bounds_grid, 256, 0, pts, n, misc, copy);
+    run(k_bounds<false>, bounds_grid, 256, 0, pts, n, misc, copy, 0u);
     run(k_morton<kSortRounds, false>, tiles, kSortThreads, 0, pts, n, misc, keys[0], counts, tiles, 1, ClearRows{});
     if (run.error != cudaSuccess) return run.error;
     return radix_sort<kSortRounds>(keys, vals, n, 30, counts, partials, s, out, true, true, nullptr, nullptr, &fin);
@@ -1160,7 +1219,7 @@ cudaError_t launch_reorder(uint4* pts, uint32_t n, uint64_t seed, int mode, void
   // pass leaves them in keys[0] (the low halves are no longer needed), which
   // frees the region for the record copy.  Then the high halves are sorted,
   // and that sort's last pass moves the records.
-  run(k_bounds<false>, bounds_grid, 256, 0, pts, n, misc, nullptr);
+  run(k_bounds<false>, bounds_grid, 256, 0, pts, n, misc, nullptr, 0u);
   run(k_morton63<kSortRounds, false>, tiles, kSortThreads, 0, pts, n, misc, keys[0], hi[0], counts, tiles, 1, ClearRows{});
   int a = 0;
   if (run.error != cudaSuccess) return run.error;

@@ -145,6 +145,7 @@ _SIGS = {
     "pcr_last_device_error": [_VP, C.POINTER(_U32)],
     "pcr_check_division": [_VP, _U32, _U32, _VP, _U32, _U32, _U32, _FLT, C.POINTER(_U64)],
     "pcr_debug_counters": [_VP, C.POINTER(_U64)],
+    "pcr_debug_fail_launch": [_INT],
     "pcr_batch_workspace_size": [C.POINTER(_U64)],
     "pcr_batch_num_configs": [C.POINTER(_INT)],
     "pcr_batch_prepare": [_VP, C.POINTER(PcrBatchCloud), _U32, C.POINTER(PcrBatchView), _U32, _FLT, _U32, _VP, _U64],

@@ -178,6 +178,7 @@ def test_release_build_has_no_counters(request):
     with pcr.Context(0, stream=torch.cuda.current_stream()) as ctx:
         out = (C.c_uint64 * 4)()
         assert pcr.lib().pcr_debug_counters(ctx.handle, out) == pcr.PCR_ERR_UNSUPPORTED
+    assert pcr.lib().pcr_debug_fail_launch(0) == pcr.PCR_ERR_UNSUPPORTED
 
 
 @pytest.fixture()
@@ -255,4 +256,37 @@ def test_debug_shuffle_with_buckets_past_shared_memory(debug_lib, oracle):
             dev = cloud.cuda()
             assert np.array_equal(reorder_gpu(c.handle, dev, n, pcr.PCR_ORDER_SHUFFLE), expect), n
             assert torch.equal(dev.cpu(), cloud[torch.from_numpy(expect)]), n
+        assert pcr.pcr_last_device_error(c.handle) == 0
+
+
+@pytest.mark.parametrize("n", (1000, 1025, 100_003, 300_007, 2_100_011, 4_100_001))
+def test_points_after_a_failed_launch(debug_lib, oracle, n):
+    """Every launch of a reorder in turn fails on the host: the call says so,
+    the Morton orders' points are untouched, the shuffle's records all there.
+    Without a failure left the call gives the oracle's order."""
+    source = scenes.random_cloud(n, seed=n % 97)
+    source[:, 3] = torch.arange(n, dtype=torch.int32)  # every record says where it came from
+    cloud, source = source.numpy(), source.cuda()
+    points = torch.empty_like(source)
+    ws = torch.empty(pcr.pcr_reorder_workspace_size(n), dtype=torch.uint8, device="cuda")
+    with pcr.Context(0, stream=torch.cuda.current_stream()) as c:
+        for mode in (pcr.PCR_ORDER_MORTON, pcr.PCR_ORDER_MORTON_SHUFFLE128, pcr.PCR_ORDER_SHUFFLE,
+                     pcr.PCR_ORDER_MORTON63, pcr.PCR_ORDER_MORTON63_SHUFFLE128):
+            for failing in range(100):
+                points.copy_(source)
+                ws.fill_(0xA5)
+                assert debug_lib.pcr_debug_fail_launch(failing) == pcr.PCR_OK
+                try:
+                    pcr.pcr_reorder_morton_shuffle128(c.handle, points, n, 3, mode, ws)
+                except pcr.PcrError as e:
+                    assert e.status == pcr.PCR_ERR_CUDA
+                else:
+                    break
+                if mode == pcr.PCR_ORDER_SHUFFLE:
+                    assert torch.equal(points[points[:, 3].argsort()], source), failing
+                else:
+                    assert torch.equal(points, source), (mode, failing)
+            debug_lib.pcr_debug_fail_launch(-1)
+            assert 0 < failing < 99
+            assert np.array_equal(points.cpu().numpy(), oracle.gather(cloud, oracle.reorder(cloud, 3, mode))), mode
         assert pcr.pcr_last_device_error(c.handle) == 0
