@@ -60,7 +60,15 @@ constexpr uint32_t kPartTile = kPartThreads * kPartRounds;
 constexpr int kMaxPassBits = 11;
 // Up to this many buckets, one pass splits them all (2.1M records with
 // their permutation: 97 us, in two passes 128).
+// Debug builds split batch orders (no records) in two passes from 9 buckets on,
+// 2.03M points, where release builds take 520M.
+#ifdef PCR_DEBUG
+template <bool REC>
+constexpr uint32_t kOnePassBuckets = REC ? 1u << kMaxPassBits : 8u;
+#else
+template <bool REC>
 constexpr uint32_t kOnePassBuckets = 1u << kMaxPassBits;
+#endif
 // Buckets of about 2000 elements, four blocks of 256 threads per SM; twice
 // that with 512 threads measured within 2% (50M: 1.59 and 1.63 ms, 400M:
 // 13.9 and 13.8).
@@ -85,10 +93,11 @@ struct RandomSplit {
   int second;
 };
 
+template <bool REC>
 constexpr RandomSplit random_split(uint32_t count) {
   const uint32_t buckets = count / kBucketMean + (count % kBucketMean != 0);
   if (buckets <= 1) return {0, 1u, 0};
-  if (buckets <= kOnePassBuckets) return {1, buckets, 0};
+  if (buckets <= kOnePassBuckets<REC>) return {1, buckets, 0};
   int bits = 0;
   while ((buckets - 1) >> bits) ++bits;
   return {2, buckets, bits / 2};
@@ -97,15 +106,16 @@ constexpr RandomSplit random_split(uint32_t count) {
 // Digits of each pass.
 constexpr uint32_t first_digits(RandomSplit p) { return ((p.buckets - 1) >> p.second) + 1; }
 constexpr uint32_t second_digits(RandomSplit p) { return 1u << p.second; }
-static_assert(first_digits(random_split(0xFFFFFFFFu)) <= 1u << kMaxPassBits &&
-                  second_digits(random_split(0xFFFFFFFFu)) <= 1u << kMaxPassBits,
+static_assert(first_digits(random_split<true>(0xFFFFFFFFu)) <= 1u << kMaxPassBits &&
+                  second_digits(random_split<true>(0xFFFFFFFFu)) <= 1u << kMaxPassBits,
               "both digits of the largest split fit a pass");
 
 // First counter of the second pass (a multiple of four words), and the words
 // of counters a split needs.
 constexpr uint64_t second_counters(RandomSplit p) { return (first_digits(p) + 3u) & ~3u; }
+template <bool REC>
 constexpr uint64_t random_counter_words(uint32_t count) {
-  const RandomSplit p = random_split(count);
+  const RandomSplit p = random_split<REC>(count);
   return p.passes == 0 ? 0 : second_counters(p) + (p.passes == 2 ? p.buckets : 0);
 }
 
@@ -439,11 +449,11 @@ __global__ void __launch_bounds__(kFinishThreads, 4)
 
 // Random order of n records in `pts` (REC; `copy` holds as many), or of n
 // indices: see RandomOut.  idx: two buffers of n words; counters:
-// random_counter_words(n) words, 16-byte aligned; partials: as exclusive_scan.
+// random_counter_words<REC>(n) words, 16-byte aligned; partials: as exclusive_scan.
 template <bool REC>
 cudaError_t random_order(uint4* pts, uint4* copy, uint32_t n, uint64_t seed, uint32_t* const idx[2],
                          uint32_t* counters, uint32_t* partials, RandomOut out, cudaStream_t s, const Device& d) {
-  const RandomSplit p = random_split(n);
+  const RandomSplit p = random_split<REC>(n);
   LaunchChain run{s};
   // The limit belongs to the kernel, for every stream and host thread: always
   // the most any size asks for.  A limit per call (98 to 115 KB by the digits)
@@ -457,7 +467,7 @@ cudaError_t random_order(uint4* pts, uint4* copy, uint32_t n, uint64_t seed, uin
   const uint32_t* iin = nullptr;
   uint32_t* ends = nullptr;
   if (p.passes > 0) {
-    const uint64_t words = random_counter_words(n);
+    const uint64_t words = random_counter_words<REC>(n);
     const uint32_t tiles = static_cast<uint32_t>((static_cast<uint64_t>(n) + kPartTile - 1) / kPartTile);
     const uint32_t radix = first_digits(p);
     uint32_t* first = counters;

@@ -259,6 +259,22 @@ def test_debug_shuffle_with_buckets_past_shared_memory(debug_lib, oracle):
         assert pcr.pcr_last_device_error(c.handle) == 0
 
 
+@pytest.mark.parametrize("n", (600_001, 2_100_011))
+def test_debug_batch_order_with_buckets_past_shared_memory(debug_lib, oracle, n):
+    """The same for the order of the 128-point batches, which moves no records
+    and writes each batch's slot: 4688 batches in 3 buckets (one partition
+    pass), and 16407 in 9, which debug builds split in two passes."""
+    from gpu_helpers import reorder_gpu
+    cloud = scenes.random_cloud(n, seed=5).numpy()
+    with pcr.Context(0, stream=torch.cuda.current_stream()) as c:
+        for mode in (pcr.PCR_ORDER_MORTON_SHUFFLE128, pcr.PCR_ORDER_MORTON63_SHUFFLE128):
+            expect = oracle.reorder(cloud, n, mode)
+            dev = torch.from_numpy(cloud.copy()).cuda()
+            assert np.array_equal(reorder_gpu(c.handle, dev, n, mode), expect), mode
+            assert np.array_equal(dev.cpu().numpy(), oracle.gather(cloud, expect)), mode
+        assert pcr.pcr_last_device_error(c.handle) == 0
+
+
 @pytest.mark.parametrize("n", (1000, 1025, 100_003, 300_007, 2_100_011, 4_100_001))
 def test_points_after_a_failed_launch(debug_lib, oracle, n):
     """Every launch of a reorder in turn fails on the host: the call says so,

@@ -148,8 +148,10 @@ def test_shuffle_at_its_pass_limits(r, oracle, n):
 @pytest.mark.parametrize("n", [255, 1023, 1024, 1025, 2049, 128 * 1024, 128 * 1024 + 1, 256 * 3072, 256 * 3072 + 1,
                                384 * 6144, 384 * 6144 + 1])
 def test_reorder_at_the_limits_of_small_sorts(r, oracle, n):
-    """One tile and two, the last size of each tile size, and the first that
-    takes the three-kernel passes; half of the points lie on few cells."""
+    """One tile and two, the last size of each small tile size and the first of
+    the next, the first that takes the three-kernel passes (256 * 3072 + 1),
+    and whole tiles of those passes and one point more; half of the points lie
+    on few cells."""
     rng = np.random.default_rng(n)
     cloud = scenes.random_cloud(n, seed=n).numpy()
     dense = rng.random(n) < 0.5
