@@ -346,23 +346,26 @@ REORDER_ALGORITHMIC_BYTES_PER_POINT = {
 #   first sort (whose last pass writes no keys).  The last pass of the sort
 #   that orders the records writes no key and no index: it moves each record
 #   from the copy to its final position (16 read, 16 written).  Batch sort and
-#   batch slots about 1; separate record copy (63-bit orders) 16 + 16.  The
-#   shuffle's entry is that of four stable passes, the form it had: 4-byte
-#   random keys written, then per pass 4 read (histogram; not the first) and
-#   key and record moved (20 read, 20 written; the last writes no key).
+#   batch slots about 1; separate record copy (63-bit orders) 16 + 16.  Morton
+#   orders of up to 786k points, which stay in the L2, take other passes.
+#   The shuffle's is shuffle_bytes_per_point.
 REORDER_BYTES_PER_POINT = {
     "morton": 32 + 20 + 4 * 20 - 8 - 8 + 32,
     "morton_shuffle128": 32 + 20 + 4 * 20 - 8 - 8 + 32 + 1,
-    "shuffle": 4 + 4 * (4 + 40) - 4 - 4,
     "morton63": 16 + 24 + 4 * 28 - 8 - 4 + 32 + 4 * 20 - 8 + 32,
     "morton63_shuffle128": 16 + 24 + 4 * 28 - 8 - 4 + 32 + 4 * 20 - 8 + 32 + 1,
 }
 
-# What the shuffle moves as partition passes (above 4.1M points, two of them):
-# first 16 read and 20 written (index and record), 4 read to count the
-# second's buckets, 20 read and 20 written, and the buckets' sort 20 read and
-# 16 written.  This is the count that is reported.
-SHUFFLE_PARTITION_BYTES_PER_POINT = 16 + 20 + 4 + 20 + 20 + 20 + 16
+
+def shuffle_bytes_per_point(n: int) -> int:
+    """DRAM bytes per point of the shuffle: the first partition reads the
+    records (16) and writes them with their indices (20), the second, above
+    2048 buckets of 1984 points, reads the indices to count its buckets (4)
+    and moves both (20 + 20), and the buckets' sort reads both (20; without a
+    partition the records alone) and writes the records (16)."""
+    if n <= 1984:
+        return 16 + 16
+    return 16 + 20 + (4 + 20 + 20 if n > 2048 * 1984 else 0) + 20 + 16
 
 
 def reorder_roofline(reorder_ms: dict, n: int, peak: float) -> dict:
@@ -371,7 +374,7 @@ def reorder_roofline(reorder_ms: dict, n: int, peak: float) -> dict:
     out = {}
     for name, ms in reorder_ms.items():
         gb = REORDER_ALGORITHMIC_BYTES_PER_POINT[name] * n / 1e9
-        own = SHUFFLE_PARTITION_BYTES_PER_POINT if name == "shuffle" else REORDER_BYTES_PER_POINT[name]
+        own = shuffle_bytes_per_point(n) if name == "shuffle" else REORDER_BYTES_PER_POINT[name]
         design_gb = own * n / 1e9
         out[name] = {"ms": ms, "algorithmic_gb": gb, "achieved_gbs": gb / (ms * 1e-3), "frac": gb / (ms * 1e-3) / peak,
                      "design_gb": design_gb, "design_over_algorithmic": design_gb / gb,
@@ -878,8 +881,8 @@ def vertex_order(h, pcr, clouds, dev) -> None:
 
 def run_batched(h, pcr, stream, dev, reps: int) -> dict:
     """8 boxes clouds (1M..200M points) x 8 orbit views (256^2..2048^2), basic
-    and HQ frames: every view through the single-view calls (7 launches per
-    view) against the batch, tuned (L2 budget and launch configuration) and
+    and HQ frames: every view through the single-view calls (7 or 8 launches
+    per view) against the batch, tuned (L2 budget and launch configuration) and
     replayed as one CUDA graph; outputs compared bit for bit."""
     import torch
     from paper_2104_07526_gb300 import scenes
@@ -915,10 +918,9 @@ def run_batched(h, pcr, stream, dev, reps: int) -> dict:
             pcr.pcr_resolve(h, pcr.PCR_RESOLVE_HQ, b["hq_image"], 0)
 
     per_ms = time_loop(per_request, stream, reps=reps, warm=1)
-    # per view: clear, render, resolve; clear, depth, colours, resolve.  HQ frames of screens that are large,
-    # or large enough and small beside their cloud, clear the sums in a launch of their own.
-    sizes = [(v.width * v.height, clouds[c].shape[0]) for c, v in views]
-    per_launches = sum(7 + (px >= 2**22 or (px >= 2**20 and n >= 2 * px)) for px, n in sizes)
+    before = pcr.pcr_launches()
+    per_request()
+    per_launches = pcr.pcr_launches() - before
     ws = torch.empty(pcr.pcr_batch_workspace_size(), dtype=torch.uint8, device=dev)
     flags = pcr.PCR_BATCH_BASIC | pcr.PCR_BATCH_HQ
     bclouds = [pcr.batch_cloud(c) for c in clouds]

@@ -681,6 +681,13 @@ PCR_API pcr_status pcr_check_division(pcr_ctx *ctx, uint32_t w_first, uint32_t w
                                       uint32_t c_first, uint32_t c_count, uint32_t c_step, float size,
                                       uint64_t out[5]);
 
+/* Kernels the calling host thread has launched through this library so far
+ * (render, resolve, clear, reorder and batch calls; recorded ones when they
+ * are recorded, not when their graph runs; not the self-check's).  The
+ * difference around a call is what the call launched.  Errors: PCR_ERR_ARG if
+ * count is NULL. */
+PCR_API pcr_status pcr_launches(uint64_t *count);
+
 /* Static, human-readable name of a status code. */
 PCR_API const char *pcr_status_string(pcr_status status);
 

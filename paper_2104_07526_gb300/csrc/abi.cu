@@ -803,6 +803,12 @@ pcr_status pcr_debug_counters(pcr_ctx* ctx, uint64_t out[4]) {
   return from_cuda(e);
 }
 
+pcr_status pcr_launches(uint64_t* count) {
+  if (!count) return PCR_ERR_ARG;
+  *count = pcr::launches_made;
+  return PCR_OK;
+}
+
 pcr_status pcr_debug_fail_launch(int after) {
 #ifdef PCR_DEBUG
   pcr::debug_launches_left = after;

@@ -16,6 +16,9 @@ struct Device {
   int num_sms = 0;
 };
 
+// Kernels this host thread has launched (pcr_launches).
+inline thread_local uint64_t launches_made = 0;
+
 #ifdef PCR_DEBUG
 // Launches this host thread makes before one fails (pcr_debug_fail_launch); none does below 0.
 inline thread_local int debug_launches_left = -1;
@@ -46,7 +49,8 @@ cudaError_t launch_kernel(void (*kernel)(P...), dim3 grid, unsigned threads, siz
   c.attrs = &attr;
   c.numAttrs = 1;
   const cudaError_t e = cudaLaunchKernelEx(&c, kernel, std::forward<A>(args)...);
-  if (e != cudaSuccess) cudaGetLastError();  // leave no error behind for the next call to find
+  if (e == cudaSuccess) ++launches_made;
+  else cudaGetLastError();  // leave no error behind for the next call to find
   return e;
 }
 

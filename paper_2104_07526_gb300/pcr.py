@@ -146,6 +146,7 @@ _SIGS = {
     "pcr_check_division": [_VP, _U32, _U32, _VP, _U32, _U32, _U32, _FLT, C.POINTER(_U64)],
     "pcr_debug_counters": [_VP, C.POINTER(_U64)],
     "pcr_debug_fail_launch": [_INT],
+    "pcr_launches": [C.POINTER(_U64)],
     "pcr_batch_workspace_size": [C.POINTER(_U64)],
     "pcr_batch_num_configs": [C.POINTER(_INT)],
     "pcr_batch_prepare": [_VP, C.POINTER(PcrBatchCloud), _U32, C.POINTER(PcrBatchView), _U32, _FLT, _U32, _VP, _U64],
@@ -376,6 +377,13 @@ def batch_view(matrix, width: int, height: int, cloud: int, flags: int, keys=Non
     return PcrBatchView((C.c_float * 16)(*vals), width, height, cloud, flags, _dptr(keys, "keys"),
                         _dptr(image, "image"), _dptr(hq_depth, "hq_depth"), _dptr(hq_rg, "hq_rg"),
                         _dptr(hq_ba, "hq_ba"), _dptr(hq_image, "hq_image"))
+
+
+def pcr_launches() -> int:
+    """Kernels this host thread has launched through the library so far."""
+    out = _U64(0)
+    _check(lib().pcr_launches(C.byref(out)), "pcr_launches")
+    return out.value
 
 
 def pcr_batch_workspace_size() -> int:

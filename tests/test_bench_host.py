@@ -60,14 +60,17 @@ def test_reorder_roofline_arithmetic():
     assert alg["morton"] == alg["morton_shuffle128"] == 128 and alg["shuffle"] == 104
     assert alg["morton63"] == alg["morton63_shuffle128"] == 192
     table = bench.REORDER_BYTES_PER_POINT
-    assert table["morton"] == 148 and table["morton_shuffle128"] == 149 and table["shuffle"] == 172
+    assert table["morton"] == 148 and table["morton_shuffle128"] == 149
     assert table["morton63"] == 276 and table["morton63_shuffle128"] == 277
+    # no partition, one, two: the limits of the library's random orders
+    assert [bench.shuffle_bytes_per_point(n) for n in (1984, 1985, 2048 * 1984, 2048 * 1984 + 1)] == [32, 72, 72, 116]
     n, peak = 800_000_000, 6760.9
     out = bench.reorder_roofline({"morton": 27.5, "shuffle": 48.0}, n, peak)
     assert out["morton"]["algorithmic_gb"] == pytest.approx(102.4)
     assert out["morton"]["achieved_gbs"] == pytest.approx(102.4 / 27.5e-3)
     assert out["morton"]["design_over_algorithmic"] == pytest.approx(148 / 128)
     assert out["shuffle"]["frac"] == pytest.approx(83.2 / 48.0e-3 / peak)
+    assert out["shuffle"]["design_over_algorithmic"] == pytest.approx(116 / 104)
 
 
 def test_cpu_sample_and_its_description():

@@ -468,6 +468,24 @@ def test_captured_frames_replay_exactly(oracle):
         pcr.pcr_capture_begin(c2.handle)  # left open: pcr_destroy drops it
 
 
+def test_launches_are_counted(r):
+    """Three launches of a basic frame, four or (sums cleared beside the depth
+    pass) five of a high-quality one, none of a call that is refused."""
+    r.upload(scenes.random_cloud(2 * 2**20, seed=1).numpy())
+
+    def launches(call):
+        before = pcr.pcr_launches()
+        call()
+        return pcr.pcr_launches() - before
+
+    for size, hq in (((1024, 1023), 4), ((1024, 1024), 5)):
+        r.view(scenes.camera((0, 0, 4), (0, 0, 0), (0, 1, 0), *size), *size)
+        assert launches(lambda: (r.render_basic(pcr.PCR_VARIANT_EARLYZ), r.resolve(pcr.PCR_RESOLVE_BASIC))) == 3
+        assert launches(lambda: (r.render_hq(pcr.PCR_VARIANT_EARLYZ), r.resolve(pcr.PCR_RESOLVE_HQ))) == hq
+    with pytest.raises(pcr.PcrError):
+        launches(lambda: pcr.pcr_render_hq(r.h, -1.0, pcr.PCR_VARIANT_EARLYZ, True))
+
+
 @pytest.mark.parametrize("scale", (1, 255, 4096, 2**24, 2**32 - 1))
 def test_hq_resolve_averages_are_exact_divisions(r, oracle, scale):
     """The resolve's reciprocal and remainder against integer division: counts

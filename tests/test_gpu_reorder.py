@@ -145,6 +145,22 @@ def test_shuffle_at_its_pass_limits(r, oracle, n):
     assert torch.equal(dev.cpu(), cloud[torch.from_numpy(expect)])
 
 
+@pytest.mark.parametrize("n", [1984, 2048 * 1984])
+def test_benchmark_counts_the_shuffles_passes(r, n):
+    """The benchmark's bytes of a shuffle change where its launches do."""
+    import bench
+
+    def launches(n):
+        points = torch.zeros((n, 4), dtype=torch.int32, device="cuda")
+        ws = torch.empty(pcr.pcr_reorder_workspace_size(n), dtype=torch.uint8, device="cuda")
+        before = pcr.pcr_launches()
+        pcr.pcr_reorder_morton_shuffle128(r.h, points, n, 0, pcr.PCR_ORDER_SHUFFLE, ws)
+        return pcr.pcr_launches() - before
+
+    assert launches(n) < launches(n + 1)
+    assert bench.shuffle_bytes_per_point(n) < bench.shuffle_bytes_per_point(n + 1)
+
+
 @pytest.mark.parametrize("n", [255, 1023, 1024, 1025, 2049, 128 * 1024, 128 * 1024 + 1, 256 * 3072, 256 * 3072 + 1,
                                384 * 6144, 384 * 6144 + 1])
 def test_reorder_at_the_limits_of_small_sorts(r, oracle, n):
