@@ -74,7 +74,8 @@ enum {
 enum {
     PCR_VARIANT_ATOMICMIN = 0,     /* Sec. 3.1: one 64-bit atomicMin per visible point */
     PCR_VARIANT_EARLYZ = 1,        /* Sec. 3.2: read the pixel first, atomic only if smaller */
-    PCR_VARIANT_DEDUP = 2,         /* Sec. 3.4: one atomic per distinct pixel per warp */
+    PCR_VARIANT_DEDUP = 2,         /* Sec. 3.4: one atomic per distinct pixel per row of 32 points;
+                                      one per point where a row's pixels are nearly all distinct */
     PCR_VARIANT_DEDUP_EARLYZ = 3,  /* Sec. 3.4 with the early test ("dedup" in Sec. 5) */
     PCR_VARIANT_REDUCE = 4,        /* Sec. 3.3: all-equal warp reduction, else pairwise */
     PCR_VARIANT_REDUCE_EARLYZ = 5, /* Sec. 3.3 with the early test */
@@ -700,7 +701,8 @@ PCR_API const char *pcr_status_string(pcr_status status);
  *   out[2] HQ colour add pairs (pcr_render_hq),
  *   out[3] early reads (Sec. 3.2) of keys and depths.
  * These show, e.g., that Sec. 3.4's deduplication sends one atomic per
- * distinct pixel per warp row.  Synchronises the stream.  Errors:
+ * distinct pixel per warp row, where it is not skipped (PCR_VARIANT_DEDUP).
+ * Synchronises the stream.  Errors:
  * PCR_ERR_UNSUPPORTED in release builds; PCR_ERR_ARG for NULL arguments;
  * PCR_ERR_CUDA if the copy fails. */
 PCR_API pcr_status pcr_debug_counters(pcr_ctx *ctx, uint64_t out[4]);

@@ -469,8 +469,9 @@ namespace {
 // framebuffer bytes fit the L2 budget (first fit, largest first); a view
 // larger than the budget gets a pass of its own.  A pass of one view shares
 // no point loads: that view goes to the phase's single-view list instead (in
-// the keys-and-depth phase, index 0, only when it asks for one frame; with
-// both, the batch pass still reads its points once for the two).
+// the keys-and-depth phase, index 0, only when it asks for one frame: with
+// both, the batch pass writes keys that serve as the depths too, where the
+// single-view calls would read the points twice).
 void build_groups(Tables* t, const pcr_batch_cloud* clouds, uint32_t num_clouds, const pcr_batch_view* views,
                   uint32_t num_views, int phase, uint64_t l2_budget) {
   uint32_t ng = 0, nord = 0, nsingle = 0;

@@ -340,10 +340,12 @@ __device__ __forceinline__ uint32_t lanemask_lt() {
 
 // In a chunk where fewer than kColorMinJoins lanes share a pixel between
 // their first two points, the lanes' slot-0 runs (four points apart) nearly
-// all lie on different pixels, and the warp step is skipped: 50M points from
-// mid distance take 0.316 ms per HQ frame with 8, 0.322 without the test and
-// 0.334 with 16; from the overview, where it rarely applies, 0.343, 0.342 and
-// 0.352.
+// all lie on different pixels, and the warp step is skipped.  HQ frames with
+// and without the test: 50M points from mid distance 299 and 309 us, 10M 86
+// and 95, 3M from inside 37 and 44; the 8 x 8 batch 19.50 and 19.91 ms.  Where
+// it rarely applies it costs up to 0.6%, in some large views more (200M boxes in
+// Morton order from mid distance 1185 and 1159 us, 800M scan 3924 and 3892).
+// A limit of 16 cost 3% where 8 costs nothing.
 constexpr int kColorMinJoins = 8;
 
 // Colour pass grouping (Listing "hqs_render" adds (r << 32 | g) and

@@ -28,7 +28,7 @@ inline thread_local int debug_launches_left = -1;
 // kernel end.  Every kernel launched so begins with after_previous() in every
 // thread, so its work starts where a plain launch's would; what overlaps is
 // the launch itself: a 1M-point frame of three launches 19.0 -> 12.3 us, 20k
-// points 11.9 -> 7.6, the seven launches of a 100k-point reorder 67 -> 48.
+// points 11.9 -> 7.6, the eight launches of a 100k-point reorder 67 -> 48.
 // No kernel lets the next one start before its own end
 // (griddepcontrol.launch_dependents), but for the clear of the high-quality
 // sums, which has something to do then: blocks that only wait stand in the way

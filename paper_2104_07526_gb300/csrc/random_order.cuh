@@ -22,7 +22,7 @@
 // comparison per pair of its elements.
 //
 // Per record the passes move 16 + 20, 4 + 20 + 20 and 20 + 16 bytes (with a
-// permutation output 4 more): 116, against 176 for four stable 8-bit passes
+// permutation output 4 more): 116, against 172 for four stable 8-bit passes
 // that carry key and record, which this replaced.  Bounds and times at 50M
 // records (ncu): the partition passes, 0.34 and 0.35 ms, are bound by their
 // shared-memory steps between barriers at 66-69% of the DRAM throughput; the

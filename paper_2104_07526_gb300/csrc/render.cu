@@ -80,7 +80,7 @@ constexpr uint32_t kFewPoints = 1u << 26;
 // Resident blocks of 256 threads per SM the kernels are compiled for (a
 // register cap: 40, or 32 for the smaller chunks): the frame is latency-bound,
 // and one resident block fewer costs more than the few instructions the cap
-// adds.  The HQ colour passes take the cap of the larger chunk.
+// adds.  The HQ colour pass takes the cap of the larger chunk.
 template <int U>
 constexpr int kMinBlocksOf = U <= kFewUnroll ? 8 : 6;
 constexpr int kHqMinBlocks = kMinBlocksOf<kUnroll>;
@@ -609,9 +609,9 @@ cudaError_t launch_clear_hq(uint32_t* depth, unsigned long long* rg, unsigned lo
 // cleared beside the pass: 4M points at 4K 120.8 -> 111.5 us, 50M at 1080p
 // 307 -> 301; below the limits 1M points at 1080p would take 33 us instead of
 // 31, 20k points at 160 x 120 11.5 instead of 10.1.  Larger clouds gain less
-// (800M at 1080p, before / beside the pass: overview 3953 / 3936 us, closeup
-// 3902 / 3883), and a view that shows none of 200M points or more loses 1 to
-// 1.7% (800M 3846 / 3886, 100M even), which the host cannot know beforehand.
+// (before / beside the pass at 1080p, 200M: overview 1038 / 1033 us, closeup
+// 992 / 985; 800M: 3925 / 3909 and 3862 / 3851); of a view that shows none of
+// the points either is faster (200M 983 / 987, 800M 3809 / 3799).
 cudaError_t launch_hq_clear_and_depth(int variant, const uint4* pts, uint32_t n, const ViewParams& v, uint32_t* depth,
                                       unsigned long long* rg, unsigned long long* ba, unsigned long long* primary,
                                       cudaStream_t s, const Device& d) {
